@@ -52,35 +52,39 @@ constexpr int kGroupLats = 64;    // members per launch (the parameter block hol
 constexpr long long kBarrierBudgetCycles = 4000000000LL;  // ~2 s at 2 GHz
 constexpr int kDefaultPersistentSteps = 32;
 
-// The collision values that follow from one lattice's nu, alpha, g beta, T0
-// and body force; the rest of RatesC<float> is shared by a launch group.
+// The values of the MRT collision (collide_x) that follow from one lattice's nu,
+// alpha, g beta, T0 and body force; the rest of RatesC<float> that it reads is
+// shared by a launch group.
 struct MemberRates {
-    float s_nu, om_nu, h_nu, h2nu, om_a, z_a, ax, hx, Fy0, g_beta, T_ref;
+    float s_nu4, om_nu4, h_nu2, nh_nu, om_a, z_a, hx, hFy0, hg_beta, T_ref;
 };
 
 inline MemberRates member_rates(const RatesC<float> &r) {
-    return MemberRates{r.s_nu, r.om_nu, r.h_nu, r.h2nu, r.om_a, r.z_a, r.ax, r.hx, r.Fy0, r.g_beta, r.T_ref};
+    return MemberRates{r.s_nu4, r.om_nu4, r.h_nu2, r.nh_nu, r.om_a, r.z_a, r.hx, r.hFy0, r.hg_beta, r.T_ref};
 }
 
 __host__ __device__ __forceinline__ void apply_member(RatesC<float> &r, const MemberRates &v) {
-    r.s_nu = v.s_nu;
-    r.om_nu = v.om_nu;
-    r.h_nu = v.h_nu;
-    r.h2nu = v.h2nu;
+    r.s_nu4 = v.s_nu4;
+    r.ns_nu4 = -v.s_nu4;
+    r.om_nu4 = v.om_nu4;
+    r.h_nu2 = v.h_nu2;
+    r.nh_nu = v.nh_nu;
     r.om_a = v.om_a;
     r.z_a = v.z_a;
-    r.ax = v.ax;
     r.hx = v.hx;
-    r.Fy0 = v.Fy0;
-    r.g_beta = v.g_beta;
+    r.hFy0 = v.hFy0;
+    r.hg_beta = v.hg_beta;
     r.T_ref = v.T_ref;
 }
 
 // Whether two lattices' rates agree outside their member-specific values.
 inline bool same_shared_rates(RatesC<float> a, RatesC<float> b) {
     const MemberRates z{};
-    apply_member(a, z);
-    apply_member(b, z);
+    for (RatesC<float> *r : {&a, &b}) {
+        apply_member(*r, z);
+        // unfolded forms of the same member values, which collide_x does not read
+        r->ns_nu4 = r->s_nu = r->om_nu = r->h_nu = r->ax = r->Fy0 = r->g_beta = 0.f;
+    }
     return std::memcmp(&a, &b, sizeof a) == 0;
 }
 

@@ -86,14 +86,18 @@ struct Ld<__half, NC> {
 // host side of the launcher.
 template <typename C>
 struct RatesC {
-    C om_e, om_nu, om_q, om_eps;  // 1 - s_k
-    C s_e, s_nu, s_q, s_eps;      // s_k
-    C h_e, h_nu, h_eps;           // 1 - s_k / 2
-    C om_a, z_a, om_ze, zv_e, om_zn;  // thermal: 1 - zeta_alpha, zeta_alpha, 1 - zeta_e, zeta_e varpi, 1 - zeta_nu
+    C om_nu, s_nu, h_nu;          // 1 - s_nu, s_nu, 1 - s_nu / 2
+    C om_a, z_a, om_ze, om_zn;    // thermal: 1 - zeta_alpha, zeta_alpha, 1 - zeta_e, 1 - zeta_nu
     C ax, Fy0, g_beta;            // F = (ax, Fy0 + g_beta (T - T_ref))
     C T_ref;
-    C hx;                         // ax / 2
-    C h2e, h2nu, h23eps;          // 2 (1 - s_e/2), 2 (1 - s_nu/2), (2/3)(1 - s_eps/2)
+    // MRT collision with M^-1's exact scalings folded in (collide_x). Quarters of 1 - s_k, of s_k, of
+    // 1 - zeta_k and of zeta_e varpi; halves of s_q, of 1 - s_nu/2 and of the force; negatives
+    // (n-) where the collision forms the negated moment
+    C om_e4, om_nu4, om_q4, om_eps4;
+    C s_e4, s_nu4, ns_nu4, s_q2, s_eps4;
+    C h_e, h_nu2, nh_nu, h3eps;   // 1 - s_e/2, (1 - s_nu/2)/2, -(1 - s_nu/2), (1 - s_eps/2)/3
+    C om_ze4, zv_e4, om_zn4;
+    C hx, hFy0, hg_beta;          // ax / 2, Fy0 / 2, g_beta / 2
     C varpi;                      // Eq. 28
     // D2Q9 temperature model (Eqs. 31-33): zeta_e, zeta_nu, zeta_q, zeta_eps and theta
     C z_e, z_nu, om_zq, z_q, om_zeps, z_eps, theta;
@@ -102,30 +106,38 @@ struct RatesC {
 template <typename C>
 inline RatesC<C> make_rates(const KParams &p) {
     RatesC<C> r;
-    r.s_e = (C)p.s_e;
+    // every folded field is an exact power-of-two multiple of the rounded rate
+    const C q = (C)0.25, h = (C)0.5;
     r.s_nu = (C)p.s_nu;
-    r.s_q = (C)p.s_q;
-    r.s_eps = (C)p.s_eps;
-    r.om_e = (C)(1.0 - p.s_e);
     r.om_nu = (C)(1.0 - p.s_nu);
-    r.om_q = (C)(1.0 - p.s_q);
-    r.om_eps = (C)(1.0 - p.s_eps);
-    r.h_e = (C)(1.0 - 0.5 * p.s_e);
     r.h_nu = (C)(1.0 - 0.5 * p.s_nu);
-    r.h_eps = (C)(1.0 - 0.5 * p.s_eps);
     r.om_a = (C)(1.0 - p.z_a);
     r.z_a = (C)p.z_a;
     r.om_ze = (C)(1.0 - p.z_e);
-    r.zv_e = (C)(p.z_e * p.varpi);
     r.om_zn = (C)(1.0 - p.z_nu);
     r.ax = (C)p.ax;
     r.Fy0 = (C)(p.ay + p.g_beta * (p.T_ref - p.T0));
     r.g_beta = (C)p.g_beta;
     r.T_ref = (C)p.T_ref;
-    r.hx = (C)(0.5 * p.ax);
-    r.h2e = (C)(2.0 * (1.0 - 0.5 * p.s_e));
-    r.h2nu = (C)(2.0 * (1.0 - 0.5 * p.s_nu));
-    r.h23eps = (C)(2.0 / 3.0 * (1.0 - 0.5 * p.s_eps));
+    r.om_e4 = q * (C)(1.0 - p.s_e);
+    r.om_nu4 = q * r.om_nu;
+    r.om_q4 = q * (C)(1.0 - p.s_q);
+    r.om_eps4 = q * (C)(1.0 - p.s_eps);
+    r.s_e4 = q * (C)p.s_e;
+    r.s_nu4 = q * r.s_nu;
+    r.ns_nu4 = -r.s_nu4;
+    r.s_q2 = h * (C)p.s_q;
+    r.s_eps4 = q * (C)p.s_eps;
+    r.h_e = (C)(1.0 - 0.5 * p.s_e);
+    r.h_nu2 = h * r.h_nu;
+    r.nh_nu = -r.h_nu;
+    r.h3eps = h * (C)(2.0 / 3.0 * (1.0 - 0.5 * p.s_eps));
+    r.om_ze4 = q * r.om_ze;
+    r.zv_e4 = q * (C)(p.z_e * p.varpi);
+    r.om_zn4 = q * r.om_zn;
+    r.hx = h * r.ax;
+    r.hFy0 = h * r.Fy0;
+    r.hg_beta = h * r.g_beta;
     r.varpi = (C)p.varpi;
     r.z_e = (C)p.z_e;
     r.z_nu = (C)p.z_nu;
@@ -357,142 +369,13 @@ __device__ __forceinline__ void nee_rebuild(const S *const *src, const Geom &g,
     }
 }
 
-// Flow collision (Eq. 8 with Eqs. 16, 17, 20 under the incompressible reading,
-// rho0 = 1) and temperature collision (Eq. 24 with Eqs. 28, 29), in place.
-// D2Q9 temperature model (Eqs. 31-33, reading: the transformation is M of
-// Eq. 13): n = M g on pair sums, n* = n - Q (n - n_eq) with n_eq = M g_eq of
-// Eq. 31 in the storage frame, g = M^-1 n*. n0 = T - T_ref is given.
-template <typename C>
-__device__ __forceinline__ void thermal_q9(const RatesC<C> &r, C t[9], C n0, C ux, C uy, C uu) {
-    const C b13 = t[1] + t[3], e13 = t[1] - t[3];
-    const C b24 = t[2] + t[4], e24 = t[2] - t[4];
-    const C b57 = t[5] + t[7], e57 = t[5] - t[7];
-    const C b68 = t[6] + t[8], e68 = t[6] - t[8];
-    const C Dt = b57 + b68;
-    const C n6 = e57 + e68, n7 = e57 - e68;
-    const C n1 = e13 + n7, n2 = e24 + n6;
-    const C n3 = (b13 + b24) + (Dt + Dt);
-    const C n4 = b13 - b24, n5 = b57 - b68, n8 = Dt;
-    const C T = r.T_ref + n0;
-    const C q1 = r.om_a * n1 + r.z_a * (T * ux);
-    const C q2 = r.om_a * n2 + r.z_a * (T * uy);
-    const C q3 = r.om_ze * n3 + r.z_e * (C(2.0 / 3.0) * n0 + r.theta * (T * uu));
-    const C q4 = r.om_zn * n4 + r.z_nu * (r.theta * (T * (ux * ux - uy * uy)));
-    const C q5 = r.om_zn * n5 + r.z_nu * (r.theta * (T * (ux * uy)));
-    const C q6 = r.om_zq * n6 + r.z_q * (C(1.0 / 3.0) * (T * uy));
-    const C q7 = r.om_zq * n7 + r.z_q * (C(1.0 / 3.0) * (T * ux));
-    const C q8 = r.om_zeps * n8 + r.z_eps * (C(1.0 / 9.0) * n0 + C(1.0 / 3.0) * (r.theta * (T * uu)));
-    const C A = C(0.25) * q3 - C(0.5) * q8;
-    const C B = C(0.25) * q4;
-    const C h1 = C(0.5) * (q1 - q7);
-    const C h2 = C(0.5) * (q2 - q6);
-    const C P = C(0.25) * (q8 + q5);
-    const C Q = C(0.25) * (q6 + q7);
-    const C R = C(0.25) * (q8 - q5);
-    const C Sx = C(0.25) * (q6 - q7);
-    t[0] = (n0 - q3) + q8;
-    t[1] = (A + B) + h1;
-    t[3] = (A + B) - h1;
-    t[2] = (A - B) + h2;
-    t[4] = (A - B) - h2;
-    t[5] = P + Q;
-    t[7] = P - Q;
-    t[6] = R + Sx;
-    t[8] = R - Sx;
-}
+// ------------------------------------------------ collisions, explicit rounding
 
-template <typename C, int TQ = 5>
-__device__ __forceinline__ void collide(const RatesC<C> &r, C f[9], C t[TQ]) {
-    // temperature first: the buoyancy of Eq. 4 needs it
-    C n0;
-    if constexpr (TQ == 9) n0 = (((t[0] + t[1]) + (t[2] + t[3])) + (t[4] + t[5])) + ((t[6] + t[7]) + t[8]);
-    else n0 = ((t[0] + t[1]) + (t[2] + t[3])) + t[4];  // T - T_ref
-    const C Fx = r.ax;
-    const C Fy = r.Fy0 + r.g_beta * n0;  // Eq. 4
-
-    // ---- D2Q9 forward map m = M f (Eq. 13) on pair sums
-    const C a13 = f[1] + f[3], d13 = f[1] - f[3];
-    const C a24 = f[2] + f[4], d24 = f[2] - f[4];
-    const C a57 = f[5] + f[7], d57 = f[5] - f[7];
-    const C a68 = f[6] + f[8], d68 = f[6] - f[8];
-    const C D = a57 + a68;
-    const C m0 = (f[0] + (a13 + a24)) + D;  // rho - rho_ref
-    const C m6 = d57 + d68;
-    const C m7 = d57 - d68;
-    const C jx = d13 + m7;
-    const C jy = d24 + m6;
-    const C m3 = (a13 + a24) + (D + D);
-    const C m4 = a13 - a24;
-    const C m5 = a57 - a68;
-    const C m8 = D;
-
-    // Eq. 19 with rho0 = 1
-    const C ux = jx + C(0.5) * Fx;
-    const C uy = jy + C(0.5) * Fy;
-    const C uu = ux * ux + uy * uy;
-    const C uF = ux * Fx + uy * Fy;
-
-    // ---- Eq. 8: m* = (1 - s) m + s m_eq + (1 - s/2) S~
-    const C p1 = jx + Fx;  // any s1: conserved moment plus the force impulse
-    const C p2 = jy + Fy;
-    const C p3 = r.om_e * m3 + r.s_e * (C(2.0 / 3.0) * m0 + uu) + r.h_e * (C(2) * uF);
-    const C p4 = r.om_nu * m4 + r.s_nu * (ux * ux - uy * uy) + r.h_nu * (C(2) * (ux * Fx - uy * Fy));
-    const C p5 = r.om_nu * m5 + r.s_nu * (ux * uy) + r.h_nu * (ux * Fy + uy * Fx);
-    // s_q m_eq + (1 - s_q/2) S~ for q_xxy, q_xyy reduces to (s_q j + F) / 3
-    const C p6 = r.om_q * m6 + C(1.0 / 3.0) * (r.s_q * jy + Fy);
-    const C p7 = r.om_q * m7 + C(1.0 / 3.0) * (r.s_q * jx + Fx);
-    const C p8 = r.om_eps * m8 + r.s_eps * (C(1.0 / 9.0) * m0 + C(1.0 / 3.0) * uu) + r.h_eps * (C(2.0 / 3.0) * uF);
-
-    // ---- back map f = M^-1 m* (Eq. A1)
-    const C A = C(0.25) * p3 - C(0.5) * p8;
-    const C B = C(0.25) * p4;
-    const C h1 = C(0.5) * (p1 - p7);
-    const C h2 = C(0.5) * (p2 - p6);
-    const C P = C(0.25) * (p8 + p5);
-    const C Q = C(0.25) * (p6 + p7);
-    const C R = C(0.25) * (p8 - p5);
-    const C Sx = C(0.25) * (p6 - p7);
-    f[0] = (m0 - p3) + p8;
-    f[1] = (A + B) + h1;
-    f[3] = (A + B) - h1;
-    f[2] = (A - B) + h2;
-    f[4] = (A - B) - h2;
-    f[5] = P + Q;
-    f[7] = P - Q;
-    f[6] = R + Sx;
-    f[8] = R - Sx;
-
-    if constexpr (TQ == 9) {
-        thermal_q9<C>(r, t, n0, ux, uy, uu);
-        return;
-    } else {
-    // ---- D2Q5: n = N g (Eq. 26), relaxation (Eq. 24) with n_eq = (T, ux T, uy T, varpi T, 0),
-    // g = N^-1 n* (Eq. A2)
-    const C n1 = t[1] - t[3];
-    const C n2 = t[2] - t[4];
-    const C n3 = (t[1] + t[3]) + (t[2] + t[4]);
-    const C n4 = (t[1] + t[3]) - (t[2] + t[4]);
-    const C T = r.T_ref + n0;
-    const C q1 = r.om_a * n1 + r.z_a * (ux * T);
-    const C q2 = r.om_a * n2 + r.z_a * (uy * T);
-    const C q3 = r.om_ze * n3 + r.zv_e * n0;
-    const C q4 = r.om_zn * n4;
-    const C c3 = C(0.25) * q3, c4 = C(0.25) * q4;
-    t[0] = n0 - q3;
-    t[1] = (c3 + c4) + C(0.5) * q1;
-    t[3] = (c3 + c4) - C(0.5) * q1;
-    t[2] = (c3 - c4) + C(0.5) * q2;
-    t[4] = (c3 - c4) - C(0.5) * q2;
-    }
-}
-
-// ------------------------------------------- FP32 collision, explicit rounding
-
-// Correctly rounded FP32 operations on one value (float) or on a pair of
-// values in one packed instruction (float2, the sm_100+ FFMA2/FADD2/FMUL2
-// path). The FP32/FP16 kernels all collide through collide_x, either per cell
-// or per pair of cells, with the same sequence of operations, so every kernel
-// variant produces the same bits.
+// Correctly rounded operations on one value (float, double) or on a pair of
+// FP32 values in one packed instruction (float2, the sm_100+ FFMA2/FADD2/FMUL2
+// path). Every kernel collides through collide_x, per cell or per pair of
+// cells, with the same sequence of operations, so every kernel variant
+// produces the same bits.
 template <typename T>
 struct Ops;
 
@@ -529,10 +412,14 @@ struct Ops<double> {
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 };
 
-// thermal_q9 with every rounding explicit (T is float or float2).
-template <typename T>
-__device__ __forceinline__ void thermal_q9_x(const RatesC<float> &r, T t[9], T n0, T ux, T uy, T uu) {
+// D2Q9 temperature model (Eqs. 31-33, reading: the transformation is M of
+// Eq. 13): n = M g on pair sums, n* = n - Q (n - n_eq) with n_eq = M g_eq of
+// Eq. 31 in the storage frame, g = M^-1 n*. n0 = T - T_ref is given.
+template <typename T, typename R>
+__device__ __forceinline__ void thermal_q9_x(const R &r, T t[9], T n0, T ux, T uy, T uu) {
     using O = Ops<T>;
+    using V = typename O::V;
+    constexpr V kThird = (V)1 / (V)3, kTwoThirds = (V)2 / (V)3, kNinth = (V)1 / (V)9;
     const T b13 = O::add(t[1], t[3]), e13 = O::sub(t[1], t[3]);
     const T b24 = O::add(t[2], t[4]), e24 = O::sub(t[2], t[4]);
     const T b57 = O::add(t[5], t[7]), e57 = O::sub(t[5], t[7]);
@@ -546,22 +433,22 @@ __device__ __forceinline__ void thermal_q9_x(const RatesC<float> &r, T t[9], T n
     const T Tuu = O::mul(O::bc(r.theta), O::mul(Tm, uu));
     const T q1 = O::fma(O::bc(r.om_a), n1, O::mul(O::bc(r.z_a), O::mul(Tm, ux)));
     const T q2 = O::fma(O::bc(r.om_a), n2, O::mul(O::bc(r.z_a), O::mul(Tm, uy)));
-    const T q3 = O::fma(O::bc(r.om_ze), n3, O::mul(O::bc(r.z_e), O::fma(O::bc(2.0f / 3.0f), n0, Tuu)));
-    const T dxy = O::fma(ux, ux, O::mul(O::bc(-1.f), O::mul(uy, uy)));
+    const T q3 = O::fma(O::bc(r.om_ze), n3, O::mul(O::bc(r.z_e), O::fma(O::bc(kTwoThirds), n0, Tuu)));
+    const T dxy = O::fma(ux, ux, O::mul(O::bc(-1), O::mul(uy, uy)));
     const T q4 = O::fma(O::bc(r.om_zn), n4, O::mul(O::bc(r.z_nu), O::mul(O::bc(r.theta), O::mul(Tm, dxy))));
     const T q5 = O::fma(O::bc(r.om_zn), n5, O::mul(O::bc(r.z_nu), O::mul(O::bc(r.theta), O::mul(Tm, O::mul(ux, uy)))));
-    const T q6 = O::fma(O::bc(r.om_zq), n6, O::mul(O::bc(r.z_q), O::mul(O::bc(1.0f / 3.0f), O::mul(Tm, uy))));
-    const T q7 = O::fma(O::bc(r.om_zq), n7, O::mul(O::bc(r.z_q), O::mul(O::bc(1.0f / 3.0f), O::mul(Tm, ux))));
+    const T q6 = O::fma(O::bc(r.om_zq), n6, O::mul(O::bc(r.z_q), O::mul(O::bc(kThird), O::mul(Tm, uy))));
+    const T q7 = O::fma(O::bc(r.om_zq), n7, O::mul(O::bc(r.z_q), O::mul(O::bc(kThird), O::mul(Tm, ux))));
     const T q8 = O::fma(O::bc(r.om_zeps), Dt,
-                        O::mul(O::bc(r.z_eps), O::fma(O::bc(1.0f / 9.0f), n0, O::mul(O::bc(1.0f / 3.0f), Tuu))));
-    const T A = O::fma(O::bc(0.25f), q3, O::mul(O::bc(-0.5f), q8));
-    const T B = O::mul(O::bc(0.25f), q4);
-    const T h1 = O::mul(O::bc(0.5f), O::sub(q1, q7));
-    const T h2 = O::mul(O::bc(0.5f), O::sub(q2, q6));
-    const T P = O::mul(O::bc(0.25f), O::add(q8, q5));
-    const T Q = O::mul(O::bc(0.25f), O::add(q6, q7));
-    const T R = O::mul(O::bc(0.25f), O::sub(q8, q5));
-    const T Sx = O::mul(O::bc(0.25f), O::sub(q6, q7));
+                        O::mul(O::bc(r.z_eps), O::fma(O::bc(kNinth), n0, O::mul(O::bc(kThird), Tuu))));
+    const T A = O::fma(O::bc((V)0.25), q3, O::mul(O::bc((V)-0.5), q8));
+    const T B = O::mul(O::bc((V)0.25), q4);
+    const T h1 = O::mul(O::bc((V)0.5), O::sub(q1, q7));
+    const T h2 = O::mul(O::bc((V)0.5), O::sub(q2, q6));
+    const T P = O::mul(O::bc((V)0.25), O::add(q8, q5));
+    const T Q = O::mul(O::bc((V)0.25), O::add(q6, q7));
+    const T Rm = O::mul(O::bc((V)0.25), O::sub(q8, q5));
+    const T Sx = O::mul(O::bc((V)0.25), O::sub(q6, q7));
     const T AB = O::add(A, B), AmB = O::sub(A, B);
     t[0] = O::add(O::sub(n0, q3), q8);
     t[1] = O::add(AB, h1);
@@ -570,24 +457,34 @@ __device__ __forceinline__ void thermal_q9_x(const RatesC<float> &r, T t[9], T n
     t[4] = O::sub(AmB, h2);
     t[5] = O::add(P, Q);
     t[7] = O::sub(P, Q);
-    t[6] = O::add(R, Sx);
-    t[8] = O::sub(R, Sx);
+    t[6] = O::add(Rm, Sx);
+    t[8] = O::sub(Rm, Sx);
 }
 
-// Same method as collide<float> (Eq. 8 with Eqs. 16, 17, 20; Eq. 24 with
-// Eqs. 28, 29; M and M^-1 of Eqs. 13 and A1 on pair sums), every rounding
-// explicit. T is float (one cell) or float2 (two cells).
-template <typename T, int TQ = 5>
-__device__ __forceinline__ void collide_x(const RatesC<float> &r, T f[9], T t[TQ]) {
+// Flow collision (Eq. 8 with Eqs. 16, 17, 20 under the incompressible reading,
+// rho0 = 1) and temperature collision (Eq. 24 with Eqs. 28, 29) in place, M and
+// M^-1 of Eqs. 13 and A1 on pair sums, every rounding explicit. T is float or
+// double (one cell) or float2 (two cells).
+//
+// The exact scalings of M^-1 and N^-1 (1/4, 1/2) are folded into the rates
+// (RatesC's quarter and half fields) and the buoyancy is carried as Fy/2, so
+// every relaxed moment comes out already scaled and the back map is additions
+// and fused multiply-adds by powers of two. A power-of-two factor moves
+// through a rounding unchanged, so the bits are those of the unscaled
+// operations; 101 FP32 operations per cell instead of 113.
+template <typename T, int TQ = 5, typename R>
+__device__ __forceinline__ void collide_x(const R &r, T f[9], T t[TQ]) {
     using O = Ops<T>;
+    using V = typename O::V;
+    constexpr V kThird = (V)1 / (V)3, kTwoThirds = (V)2 / (V)3, kNinth = (V)1 / (V)9;
     T n0;
     if constexpr (TQ == 9)
         n0 = O::add(O::add(O::add(O::add(t[0], t[1]), O::add(t[2], t[3])), O::add(t[4], t[5])),
                     O::add(O::add(t[6], t[7]), t[8]));
     else
         n0 = O::add(O::add(O::add(t[0], t[1]), O::add(t[2], t[3])), t[4]);  // T - T_ref
-    const T Fx = O::bc(r.ax);
-    const T Fy = O::fma(O::bc(r.g_beta), n0, O::bc(r.Fy0));  // Eq. 4
+    const T hFx = O::bc(r.hx);                               // F / 2 (Eq. 4)
+    const T hFy = O::fma(O::bc(r.hg_beta), n0, O::bc(r.hFy0));
     // D2Q9 forward map (Eq. 13)
     const T a13 = O::add(f[1], f[3]), d13 = O::sub(f[1], f[3]);
     const T a24 = O::add(f[2], f[4]), d24 = O::sub(f[2], f[4]);
@@ -600,54 +497,55 @@ __device__ __forceinline__ void collide_x(const RatesC<float> &r, T f[9], T t[TQ
     const T m7 = O::sub(d57, d68);
     const T jx = O::add(d13, m7);
     const T jy = O::add(d24, m6);
-    const T m3 = O::add(A4, O::add(D, D));
+    const T m3 = O::fma(O::bc(2), D, A4);
     const T m4 = O::sub(a13, a24);
     const T m5 = O::sub(a57, a68);
     // Eq. 19 with rho0 = 1
-    const T ux = O::add(jx, O::bc(r.hx));
-    const T uy = O::fma(O::bc(0.5f), Fy, jy);
+    const T ux = O::add(jx, hFx);
+    const T uy = O::add(jy, hFy);
+    const T nux = O::mul(O::bc(-1), ux);
     const T uyuy = O::mul(uy, uy);
+    const T uyFy = O::mul(uy, hFy);
     const T uu = O::fma(ux, ux, uyuy);
-    const T uF = O::fma(ux, Fx, O::mul(uy, Fy));
-    // Eq. 8
-    const T p1 = O::add(jx, Fx);
-    const T p2 = O::add(jy, Fy);
-    const T p3 = O::fma(O::bc(r.om_e), m3,
-                        O::fma(O::bc(r.s_e), O::fma(O::bc(2.0f / 3.0f), m0, uu), O::mul(O::bc(r.h2e), uF)));
-    const T dxy = O::fma(ux, ux, O::mul(O::bc(-1.f), uyuy));
-    const T dF = O::fma(ux, Fx, O::mul(O::bc(-1.f), O::mul(uy, Fy)));
-    const T p4 = O::fma(O::bc(r.om_nu), m4, O::fma(O::bc(r.s_nu), dxy, O::mul(O::bc(r.h2nu), dF)));
-    const T cF = O::fma(ux, Fy, O::mul(uy, Fx));
-    const T p5 = O::fma(O::bc(r.om_nu), m5, O::fma(O::bc(r.s_nu), O::mul(ux, uy), O::mul(O::bc(r.h_nu), cF)));
-    const T p6 = O::fma(O::bc(r.om_q), m6, O::mul(O::bc(1.0f / 3.0f), O::fma(O::bc(r.s_q), jy, Fy)));
-    const T p7 = O::fma(O::bc(r.om_q), m7, O::mul(O::bc(1.0f / 3.0f), O::fma(O::bc(r.s_q), jx, Fx)));
-    const T p8 = O::fma(O::bc(r.om_eps), D,
-                        O::fma(O::bc(r.s_eps), O::fma(O::bc(1.0f / 9.0f), m0, O::mul(O::bc(1.0f / 3.0f), uu)),
-                               O::mul(O::bc(r.h23eps), uF)));
-    // back map (Eq. A1); the 1/2 and 1/4 scalings are exact
-    const T A = O::fma(O::bc(0.25f), p3, O::mul(O::bc(-0.5f), p8));
-    const T B = O::mul(O::bc(0.25f), p4);
-    const T h1 = O::mul(O::bc(0.5f), O::sub(p1, p7));
-    const T h2 = O::mul(O::bc(0.5f), O::sub(p2, p6));
-    const T P = O::mul(O::bc(0.25f), O::add(p8, p5));
-    const T Q = O::mul(O::bc(0.25f), O::add(p6, p7));
-    const T R = O::mul(O::bc(0.25f), O::sub(p8, p5));
-    const T Sx = O::mul(O::bc(0.25f), O::sub(p6, p7));
-    const T AB = O::add(A, B), AmB = O::sub(A, B);
-    f[0] = O::add(O::sub(m0, p3), p8);
+    const T uF = O::fma(ux, hFx, uyFy);      // u.F / 2
+    const T ndxy = O::fma(nux, ux, uyuy);    // uy^2 - ux^2
+    const T ndF = O::fma(nux, hFx, uyFy);    // (uy Fy - ux Fx) / 2
+    const T cF = O::fma(ux, hFy, O::mul(uy, hFx));
+    // Eq. 8; p1, p2 halved, p3..p8 quartered
+    const T p1 = O::fma(O::bc((V)0.5), jx, hFx);
+    const T p2 = O::fma(O::bc((V)0.5), jy, hFy);
+    const T p3 = O::fma(O::bc(r.om_e4), m3,
+                        O::fma(O::bc(r.s_e4), O::fma(O::bc(kTwoThirds), m0, uu), O::mul(O::bc(r.h_e), uF)));
+    const T p4 = O::fma(O::bc(r.om_nu4), m4, O::fma(O::bc(r.ns_nu4), ndxy, O::mul(O::bc(r.nh_nu), ndF)));
+    const T p5 = O::fma(O::bc(r.om_nu4), m5, O::fma(O::bc(r.s_nu4), O::mul(ux, uy), O::mul(O::bc(r.h_nu2), cF)));
+    const T p6 = O::fma(O::bc(r.om_q4), m6, O::mul(O::bc(kThird / 2), O::fma(O::bc(r.s_q2), jy, hFy)));
+    const T p7 = O::fma(O::bc(r.om_q4), m7, O::mul(O::bc(kThird / 2), O::fma(O::bc(r.s_q2), jx, hFx)));
+    const T p8 = O::fma(O::bc(r.om_eps4), D,
+                        O::fma(O::bc(r.s_eps4), O::fma(O::bc(kNinth), m0, O::mul(O::bc(kThird), uu)),
+                               O::mul(O::bc(r.h3eps), uF)));
+    // back map (Eq. A1)
+    const T A = O::fma(O::bc(-2), p8, p3);
+    const T h1 = O::fma(O::bc(-2), p7, p1);
+    const T h2 = O::fma(O::bc(-2), p6, p2);
+    const T P = O::add(p8, p5);
+    const T Q = O::add(p6, p7);
+    const T Rm = O::sub(p8, p5);
+    const T Sx = O::sub(p6, p7);
+    const T AB = O::add(A, p4), AmB = O::sub(A, p4);
+    f[0] = O::fma(O::bc(4), p8, O::fma(O::bc(-4), p3, m0));
     f[1] = O::add(AB, h1);
     f[3] = O::sub(AB, h1);
     f[2] = O::add(AmB, h2);
     f[4] = O::sub(AmB, h2);
     f[5] = O::add(P, Q);
     f[7] = O::sub(P, Q);
-    f[6] = O::add(R, Sx);
-    f[8] = O::sub(R, Sx);
+    f[6] = O::add(Rm, Sx);
+    f[8] = O::sub(Rm, Sx);
     if constexpr (TQ == 9) {
         thermal_q9_x<T>(r, t, n0, ux, uy, uu);
         return;
     } else {
-    // D2Q5 forward map (Eq. 26), relaxation (Eq. 24) and back map (Eq. A2)
+    // D2Q5 forward map (Eq. 26), relaxation (Eq. 24; q3, q4 quartered) and back map (Eq. A2)
     const T s13 = O::add(t[1], t[3]), s24 = O::add(t[2], t[4]);
     const T n1 = O::sub(t[1], t[3]);
     const T n2 = O::sub(t[2], t[4]);
@@ -656,15 +554,14 @@ __device__ __forceinline__ void collide_x(const RatesC<float> &r, T f[9], T t[TQ
     const T Tm = O::add(O::bc(r.T_ref), n0);
     const T q1 = O::fma(O::bc(r.om_a), n1, O::mul(O::bc(r.z_a), O::mul(ux, Tm)));
     const T q2 = O::fma(O::bc(r.om_a), n2, O::mul(O::bc(r.z_a), O::mul(uy, Tm)));
-    const T q3 = O::fma(O::bc(r.om_ze), n3, O::mul(O::bc(r.zv_e), n0));
-    const T q4 = O::mul(O::bc(r.om_zn), n4);
-    const T c3 = O::mul(O::bc(0.25f), q3), c4 = O::mul(O::bc(0.25f), q4);
-    const T c34 = O::add(c3, c4), c3m4 = O::sub(c3, c4);
-    t[0] = O::sub(n0, q3);
-    t[1] = O::fma(O::bc(0.5f), q1, c34);
-    t[3] = O::fma(O::bc(-0.5f), q1, c34);
-    t[2] = O::fma(O::bc(0.5f), q2, c3m4);
-    t[4] = O::fma(O::bc(-0.5f), q2, c3m4);
+    const T q3 = O::fma(O::bc(r.om_ze4), n3, O::mul(O::bc(r.zv_e4), n0));
+    const T q4 = O::mul(O::bc(r.om_zn4), n4);
+    const T c34 = O::add(q3, q4), c3m4 = O::sub(q3, q4);
+    t[0] = O::fma(O::bc(-4), q3, n0);
+    t[1] = O::fma(O::bc((V)0.5), q1, c34);
+    t[3] = O::fma(O::bc((V)-0.5), q1, c34);
+    t[2] = O::fma(O::bc((V)0.5), q2, c3m4);
+    t[4] = O::fma(O::bc((V)-0.5), q2, c3m4);
     }
 }
 
@@ -769,15 +666,13 @@ __device__ __forceinline__ void collide_bgk_x(const R &r, T f[9], T t[TQ]) {
     bgk_pair<6, 8, T, R, TQ>(r, f, t, C0, ux, uy, Fx, Fy, uu, zn0, zT);
 }
 
-// The collision of one cell in the storage's compute type: MRT (exact FP64
-// operators, or explicit FP32 rounding for shifted storage) or BGK.
+// The collision of one cell in the storage's compute type: MRT or BGK.
 template <typename S, int TQ, bool BGK>
 __device__ __forceinline__ void collide_cell(const RatesC<typename Store<S>::C> &r, typename Store<S>::C f[9],
                                              typename Store<S>::C t[TQ]) {
     using C = typename Store<S>::C;
     if constexpr (BGK) collide_bgk_x<C, RatesC<C>, TQ>(r, f, t);
-    else if constexpr (Store<S>::kShifted) collide_x<float, TQ>(r, f, t);
-    else collide<C, TQ>(r, f, t);
+    else collide_x<C, TQ>(r, f, t);
 }
 
 // Collide cells K and K + 1 of an N-cell group as one float2 pair, in place.
