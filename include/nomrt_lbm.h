@@ -160,13 +160,18 @@ lbm_status lbm_validate(const lbm_params *p);
 lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, size_t device_bytes,
                       lbm_lattice **out);
 
-/* Advance nsteps >= 0 time steps (Eqs. 8-9 and 24-25, fused, one kernel per
- * step, plus one for the boundary nodes of node-based walls). Asynchronous on the
- * lattice's stream. Runs of 4 steps or more replay CUDA graphs of 32 and of 4
- * steps, captured once per step-kernel choice (the same kernels and bits,
- * without the launch gap between steps; a step launched directly first where
- * the graphs' starting buffer needs it); shorter runs and the remainder, and
- * calls on a stream that is being captured, launch the kernels directly. */
+/* Advance nsteps >= 0 time steps (Eqs. 8-9 and 24-25, fused). Asynchronous on the
+ * lattice's stream. With the AUTO step kernel, runs of two steps or more of an
+ * FP32 or FP16 lattice without node-based walls (and with at most 15 walls; in
+ * FP16 up to 600,000 cells) take up to eight steps per launch, tile by tile in
+ * shared memory, the tile and the steps per launch chosen from the lattice's
+ * size; the bits are those of single steps. Every other step is one kernel,
+ * plus one for the boundary nodes of node-based walls; runs of 4 such steps or
+ * more replay CUDA graphs of 32 and of 4 steps, captured once per step-kernel
+ * choice (the same kernels and bits, without the launch gap between steps; a
+ * step launched directly first where the graphs' starting buffer needs it);
+ * shorter runs and the remainder, and calls on a stream that is being captured,
+ * launch the kernels directly. */
 lbm_status lbm_step(lbm_lattice *h, int64_t nsteps);
 
 /* Wait for the lattice's stream. LBM_ETIMEOUT if a step kernel gave up one of
@@ -174,8 +179,9 @@ lbm_status lbm_step(lbm_lattice *h, int64_t nsteps);
 lbm_status lbm_sync(lbm_lattice *h);
 
 /* Step kernel variants. All compute the same arithmetic and give the same
- * bits for a given storage. AUTO picks the fastest measured on GB300: the
- * scalar kernel for FP64; VEC4 for FP32 / FP16 with config 1 / 1 (MRT, D2Q5),
+ * bits for a given storage. AUTO picks the fastest measured on GB300: several
+ * steps per launch where lbm_step says so, and for single steps the scalar
+ * kernel for FP64, VEC4 for FP32 / FP16 with config 1 / 1 (MRT, D2Q5),
  * 0 / 1 (BGK, D2Q5) or 0 / 0 (D2Q9 temperature model), except VEC4W config 1
  * for FP32 MRT D2Q5 lattices whose rows are not a multiple of 512 cells.
  * SCALAR: one cell per thread. VEC4: four cells per thread with 128-bit (FP32)

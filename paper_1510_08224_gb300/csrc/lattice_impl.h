@@ -58,6 +58,13 @@ struct lbm_lattice {
     bool graph_off = false;       // capture failed or the stream cannot be captured
     bool direct_done = false;     // the current kernel choice has run at least once directly
 
+    // several steps per launch (AUTO): the plan for this lattice (shape -1: none), made at the first
+    // run of two steps or more, and the tensor maps of its two buffers
+    const nomrt::TileLaunchers *tile = nullptr;
+    nomrt::TilePlan tile_plan{-1, 0};
+    bool tile_planned = false;
+    CUtensorMap tile_map[2];
+
     double *stage() const { return reinterpret_cast<double *>(mem + lay.off_stage); }
     double *partials() const { return reinterpret_cast<double *>(mem + lay.off_part); }
     double *result() const { return reinterpret_cast<double *>(mem + lay.off_res); }

@@ -463,6 +463,38 @@ lbm_status step_direct(lbm_lattice *h, int64_t n) {
     return LBM_OK;
 }
 
+// Whether h steps several times per launch (its plan and tensor maps made at the first call).
+bool plan_tiles(lbm_lattice *h) {
+    if (!h->tile_planned) {
+        h->tile_planned = true;
+        h->tile = nomrt::tile_launchers(h->storage, h->kp.tq, h->kp.bgk);
+        int dev = 0, sms = 0;
+        if (h->tile && cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+            h->tile_plan = h->tile->plan(h->kp, sms);
+        if (h->tile_plan.shape >= 0 && h->tile->maps(h->kp, h->tile_plan.shape, h->tile_map) != cudaSuccess)
+            h->tile_plan.shape = -1;
+        cudaGetLastError();
+    }
+    return h->tile_plan.shape >= 0;
+}
+
+// n >= 2 steps as evenly sized launches of at most tile_plan.steps steps. Each is a
+// programmatic dependent of the one before and costs the GPU more time than its
+// launch costs the host, so they are launched directly.
+lbm_status step_tiles(lbm_lattice *h, int64_t n) {
+    const int64_t launches = (n + h->tile_plan.steps - 1) / h->tile_plan.steps;
+    for (int64_t i = launches; i > 0; --i) {
+        const int k = (int)((n + i - 1) / i);
+        cudaError_t e = h->tile->launch(h->kp, h->tile_plan.shape, h->tile_map[h->cur], h->cur, k, h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "tile kernel");
+        h->cur ^= 1;
+        h->steps += k;
+        n -= k;
+    }
+    return LBM_OK;
+}
+
 // The device-side maps of a lattice whose walls are all halfway (no node-based
 // wall, so the layout does not depend on the flag map): one thread per cell of
 // the pitched layout reads the wall ids of the cell and of its eight pull
@@ -677,6 +709,13 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
         hw[k].adiabatic = w.kind == LBM_T_ADIABATIC ? 1.0 : 0.0;
     }
 
+    hw[0].f[9] = 1.f;
+    for (int k = 1; k <= p->n_walls; ++k) {
+        for (int i = 0; i < 9; ++i) hw[k].f[i] = (float)hw[k].cf[i], hw[k].f[11 + i] = (float)hw[k].tb9[i];
+        hw[k].f[9] = (float)hw[k].tsgn;
+        hw[k].f[10] = (float)hw[k].tb;
+    }
+
     KParams &kp = h->kp;
     kp.nx = nx;
     kp.ny = ny;
@@ -689,6 +728,9 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
     kp.mask = reinterpret_cast<const uint8_t *>(h->mem + h->lay.off_mask);
     kp.flags = reinterpret_cast<const uint8_t *>(h->mem + h->lay.off_flags);
     kp.walls = reinterpret_cast<const WallDev *>(h->mem + h->lay.off_walls);
+    kp.n_walls = p->n_walls;
+    kp.moving = 0;
+    for (int k = 0; k < p->n_walls; ++k) kp.moving |= p->walls[k].ux != 0.0 || p->walls[k].uy != 0.0;
     Derived d = derive(p);
     kp.s_e = p->s_e;
     kp.s_nu = d.s_nu;
@@ -828,6 +870,7 @@ lbm_status lbm_step(lbm_lattice *h, int64_t nsteps) {
     if (!h) return fail(nullptr, LBM_EINVAL, "lattice is NULL");
     if (nsteps < 0) return fail(h, LBM_EINVAL, "nsteps must be >= 0");
     if (h->batch) return fail(h, LBM_EINVAL, "lattice belongs to a batch: step it with lbm_batch_step");
+    if (nsteps > 1 && h->kp.variant == nomrt::kStepAuto && plan_tiles(h)) return step_tiles(h, nsteps);
     // Runs of kGraphShort steps or more replay captured graphs of kGraphSteps and kGraphShort
     // steps: the same kernels with the same arguments, without the launch gap between steps.
     // Direct launches serve short runs and remainders, a stream that is already being

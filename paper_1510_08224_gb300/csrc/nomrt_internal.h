@@ -3,6 +3,7 @@
 // kernels_f16.cu). Not part of the public ABI.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 
@@ -42,6 +43,8 @@ constexpr int kStepVec4w = 5;
 // Shapes of the TMA step kernel (see launchers.cuh).
 constexpr int kTmaConfigCount = 5;
 
+constexpr int kWallFloats = 20;
+
 // Per-wall constants, indexed by wall id (entry 0 unused). cf[i] is Ladd's
 // moving-wall term 2 w_i rho0 (e_i . u_w) / c_s^2 for direction i; a
 // temperature link from the wall gives g_i = tsgn * g*_opp(i) + tb, with
@@ -56,6 +59,7 @@ struct WallDev {
     double nee;       // 1: node-based wall (non-equilibrium extrapolation), 0: halfway
     double adiabatic; // 1: adiabatic, 0: fixed temperature
     double tb9[9];    // D2Q9 temperature model: g_i = tsgn g*_opp(i) + tb9[i]
+    float f[kWallFloats];  // cf, tsgn, tb, tb9 rounded to FP32, for the FP32 / FP16 kernels (entry 0: tsgn = 1, the rest 0)
 };
 
 // Everything a kernel needs to know about one lattice, in FP64; each kernel
@@ -68,6 +72,8 @@ struct KParams {
     const uint8_t *mask;        // link map: bit i-1 set if direction i pulls from a solid cell
     const uint8_t *flags;       // wall ids
     const WallDev *walls;
+    int n_walls;
+    int moving;                 // some halfway wall moves (a non-zero Ladd term)
     // rates and constants
     double s_e, s_nu, s_q, s_eps;     // Eq. 20
     double z_a, z_e, z_nu;            // Eq. 29
@@ -86,6 +92,23 @@ struct KParams {
     // every checked access must stay in, and the word that records the first failing check
     const char *blk_lo, *blk_hi;
     int *oob;
+};
+
+// How a lattice steps several times per launch: a tile shape (an index, -1: it
+// does not) and the steps per launch.
+struct TilePlan {
+    int shape, steps;
+};
+
+// The several-steps-per-launch kernels (tile.cuh) of one storage, temperature
+// lattice and collision.
+struct TileLaunchers {
+    // the plan for a lattice on a GPU of `sms` SMs
+    TilePlan (*plan)(const KParams &, int sms);
+    // the tensor maps of the lattice's two buffers for a shape
+    cudaError_t (*maps)(const KParams &, int shape, CUtensorMap map[2]);
+    // k <= plan.steps steps, reading buffer src (its tensor map in `map`), writing 1 - src
+    cudaError_t (*launch)(const KParams &, int shape, const CUtensorMap &map, int src, int k, cudaStream_t st);
 };
 
 // Launchers, one set per storage type (0 = f64, 1 = f32-shifted, 2 = f16-shifted).
@@ -113,6 +136,9 @@ struct Launchers {
     cudaError_t (*residual)(const KParams &, int buf, double *snap, int have_snap, double *partials,
                             cudaStream_t st);
 };
+
+// storage: the ABI's (0 f64, 1 f32, 2 f16); nullptr for FP64, which steps once per launch.
+const TileLaunchers *tile_launchers(int storage, int tq, int bgk);
 
 const Launchers &launchers_f64();
 const Launchers &launchers_f32();

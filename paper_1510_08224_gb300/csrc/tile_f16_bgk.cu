@@ -1,0 +1,10 @@
+// Several steps per launch (tile.cuh): FP16 storage, BGK collisions, D2Q5 temperature.
+#include "tile_launch.cuh"
+
+namespace nomrt {
+
+const TileLaunchers *tile_f16_bgk() {
+    return TileSet<__half, 5, true, ShapeOf<24, 24, 288, 2>, ShapeOf<32, 24, 384, 2>, ShapeOf<40, 24, 256, 3>, ShapeOf<40, 24, 128, 4>>::get();
+}
+
+}  // namespace nomrt

@@ -1,0 +1,219 @@
+// Launchers of the several-steps-per-launch kernels (tile.cuh): the tile shapes,
+// the choice of shape and steps per launch for a lattice, tensor maps.
+#pragma once
+
+#include <algorithm>
+#include <atomic>
+#include <cmath>
+
+#include "tile.cuh"
+
+namespace nomrt {
+
+struct TileShape {
+    int rx, ry, threads, per_sm;  // region, block, resident blocks asked of ptxas
+    size_t smem;
+};
+
+// Output columns and rows of a tile of a shape in a launch of k steps.
+inline int shape_cols(const TileShape &s, int k) { return (s.rx - tile_margin(k) - k) & ~3; }
+inline int shape_rows(const TileShape &s, int k) { return s.ry - 2 * k; }
+
+// The rows and columns a lattice's tiles cover: a non-periodic axis ends in a
+// frame of cells that are not updated.
+struct TileCover {
+    int row0, rows, cols;
+};
+inline TileCover tile_cover(const KParams &p) {
+    return TileCover{p.py ? 0 : 1, p.py ? p.ny : p.ny - 2, p.px ? p.nx : p.nx - 1};
+}
+
+// Estimated cycles of one launch of k steps, all its tiles: a launch's own cost,
+// then waves of resident blocks. A block's steps take at least their latency
+// (one pass of a thread over its pairs, a barrier); the blocks of an SM share
+// its pipes, better the more of them are out of step with one another; and the
+// wave's bytes take their time on the way from and to HBM (or L2, for a lattice
+// that fits it), overlapped with the steps but not entirely. The constants are
+// a least-squares fit to 200 launches on lattices of 64^2 to 4096 x 2048 cells
+// with 2 to 8 steps per launch (rms error 12 %).
+inline double tile_cycles(const TileShape &s, int k, long long tiles, double cell_bytes, bool fits_l2, int sms) {
+    constexpr double kLaunch = 9000, kBlock = 1770, kLatency = 1360, kRound = 0.7;
+    constexpr double kPairWarp[4] = {151, 110, 92, 91};  // cycles per 32 pairs with 1..4 blocks on the SM
+    constexpr double kHbm = 25.8, kL2 = 3 * kHbm;        // bytes per cycle and SM
+    auto wave = [&](int n) {
+        double steps = kBlock;
+        for (int l = 1; l <= k; ++l) {
+            const int pairs = (s.ry / 2 - l) * (l < k ? s.rx : shape_cols(s, k));
+            const int rounds = (pairs + s.threads - 1) / s.threads;
+            steps += std::max(kLatency * (1 + kRound * (rounds - 1)),
+                              n * ((pairs + 31) / 32) * kPairWarp[std::min(n, 4) - 1]);
+        }
+        const double bytes = n * shape_cols(s, k) * shape_rows(s, k) * cell_bytes / (fits_l2 ? kL2 : kHbm);
+        return std::cbrt(steps * steps * steps + bytes * bytes * bytes);
+    };
+    const long long slots = (long long)sms * s.per_sm;
+    const long long full = tiles / slots, rest = tiles % slots;
+    return kLaunch + (double)full * wave(s.per_sm) + (rest ? wave((int)((rest + sms - 1) / sms)) : 0.0);
+}
+
+constexpr int kTileMaxSteps = 8;
+constexpr long long kTileMostF16 = 600000;  // cells
+constexpr double kL2Bytes = 100e6;          // what of the 129 MB L2 two buffers can count on
+
+// The shape and steps per launch with the least estimated time per step.
+// Lattices with node-based walls or more walls than a block keeps step once per
+// launch; so do FP16 lattices whose single steps are bound by HBM (1024^2 cells:
+// 14.0 us a step against 17.4; 600^2: 9.1 against 7.9), where the FP32 images a
+// block keeps cost more than the passes over memory they save.
+inline TilePlan choose_tile(const KParams &p, int nq, int elem, const TileShape *shapes, int n_shapes, int sms) {
+    TilePlan best{-1, 0};
+    double least = 0;
+    const TileCover c = tile_cover(p);
+    if (p.n_nee > 0 || p.n_walls > kTileWalls || c.rows <= 0 || c.cols <= 0 || sms <= 0) return best;
+    if (elem == 2 && (long long)p.nx * p.ny > kTileMostF16) return best;
+    const double cell_bytes = 2.0 * nq * elem;
+    const bool fits_l2 = cell_bytes * p.nx * p.ny < kL2Bytes;
+    for (int i = 0; i < n_shapes; ++i)
+        for (int k = 2; k <= kTileMaxSteps; ++k) {
+            const int tx = shape_cols(shapes[i], k), ty = shape_rows(shapes[i], k);
+            if (tx < 4 || ty < 2) break;
+            const long long gx = (c.cols + tx - 1) / tx, gy = (c.rows + ty - 1) / ty;
+            if (gy > 65535 || gx * gy > 0x3FFFFFFF) continue;  // the launch grid's y limit
+            const double t = tile_cycles(shapes[i], k, gx * gy, cell_bytes, fits_l2, sms) / k;
+            if (best.shape < 0 || t < least) {
+                best = TilePlan{i, k};
+                least = t;
+            }
+        }
+    return best;
+}
+
+// The tensor map of buffer `buf` for regions of RX x RY cells: x, row pair, row
+// parity, plane (for an odd ny the last row pair's second row lies past the
+// plane, in the lattice's block; the kernel treats it as off the lattice).
+inline cudaError_t make_tile_map(const KParams &p, int buf, int nq, int rx, int ry, CUtensorMap *map) {
+    using Encode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static std::atomic<void *> entry{nullptr};
+    void *fn = entry.load(std::memory_order_acquire);
+    if (!fn) {
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e =
+            cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+        if (e != cudaSuccess) return e;
+        if (found != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
+        entry.store(fn, std::memory_order_release);
+    }
+    const cuuint64_t row = (cuuint64_t)p.pitch * 4;
+    const cuuint64_t dims[4] = {(cuuint64_t)p.pitch, (cuuint64_t)(p.ny + 1) / 2, 2, (cuuint64_t)nq};
+    const cuuint64_t strides[3] = {2 * row, row, (cuuint64_t)p.plane * 4};
+    const cuuint32_t box[4] = {(cuuint32_t)rx, (cuuint32_t)ry / 2, 1, (cuuint32_t)nq};
+    const cuuint32_t one[4] = {1, 1, 1, 1};
+    const CUresult r = reinterpret_cast<Encode>(fn)(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, p.pop[buf], dims, strides,
+                                                    box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// SMs of the current device, read once per device (0 if it cannot be read).
+inline int tile_sms(int dev) {
+    static std::atomic<int> sms[kMaxDevices];
+    if (dev < 0 || dev >= kMaxDevices) return 0;
+    int n = sms[dev].load(std::memory_order_relaxed);
+    if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+        sms[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
+// Dynamic shared memory of a launch of `tiles` blocks: the shape's, or, where
+// the grid fits the GPU at n blocks per SM, as much as lets no more than n
+// reside, so that the blocks spread over all SMs (as programmatic dependents
+// they would otherwise double up on the SMs the previous launch leaves first:
+// 64^2 cells, 8 steps per launch, 1.48 against 1.21 us a step).
+inline size_t tile_smem_bytes(const TileShape &s, long long tiles, int sms) {
+    constexpr size_t kSm = 227 * 1024, kPerBlock = 1024;  // shared memory per SM, and what the system takes per block
+    if (sms <= 0) return s.smem;
+    const long long n = (tiles + sms - 1) / sms;
+    if (n > s.per_sm) return s.smem;
+    return std::max(s.smem, (kSm / (size_t)n - kPerBlock - 256) & ~(size_t)1023);
+}
+
+template <typename S>
+using TileKernel = void (*)(const Planes<S>, const Geom, const RatesC<float>, const CUtensorMap, TileWalls, int, int,
+                            int, int, int *);
+
+// One launch of k steps.
+template <typename S>
+cudaError_t launch_tile(TileKernel<S> kern, const TileShape &s, std::atomic<bool> *ready, const KParams &p,
+                        const CUtensorMap &map, int src, int k, cudaStream_t st) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    if (!ready[dev].load(std::memory_order_acquire)) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return e;
+        ready[dev].store(true, std::memory_order_release);
+    }
+    const int sms = tile_sms(dev);
+    const TileCover c = tile_cover(p);
+    const int tx = shape_cols(s, k), ty = shape_rows(s, k);
+    if (tx < 4 || ty < 2) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((c.cols + tx - 1) / tx, (c.rows + ty - 1) / ty);
+    cfg.blockDim = dim3(s.threads);
+    const long long tiles = (long long)cfg.gridDim.x * cfg.gridDim.y;
+    cfg.dynamicSmemBytes = tile_smem_bytes(s, tiles, sms);
+    cfg.stream = st;
+    // a programmatic dependent of the previous launch (the kernel waits for that grid's
+    // completion before it reads a population)
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const int resident = sms * s.per_sm;
+    return cudaLaunchKernelEx(&cfg, kern, make_planes<S>(p, src), make_geom(p), make_rates<float>(p), map,
+                              TileWalls{p.n_walls, p.moving}, k, c.row0, (int)(tiles <= resident), resident, p.status);
+}
+
+// The shapes of one storage, temperature lattice and collision: region columns
+// and rows, threads, resident blocks per SM.
+template <int RX, int RY, int T, int MINB>
+struct ShapeOf {};
+
+template <typename S, int TQ, bool BGK, typename... SHAPES>
+struct TileSet;
+
+template <typename S, int TQ, bool BGK, int... RX, int... RY, int... T, int... MINB>
+struct TileSet<S, TQ, BGK, ShapeOf<RX, RY, T, MINB>...> {
+    static constexpr int N = sizeof...(RX);
+    static const TileShape *shapes() {
+        static const TileShape s[N] = {TileShape{RX, RY, T, MINB, TileLayout<TQ, RX, RY>::bytes()}...};
+        return s;
+    }
+    static TilePlan plan(const KParams &p, int sms) { return choose_tile(p, 9 + TQ, (int)sizeof(S), shapes(), N, sms); }
+    static cudaError_t maps(const KParams &p, int shape, CUtensorMap map[2]) {
+        if (shape < 0 || shape >= N) return cudaErrorInvalidValue;
+        if (sizeof(S) != 4) return cudaSuccess;  // FP16 regions are not copied through a tensor map
+        for (int b = 0; b < 2; ++b) {
+            const cudaError_t e = make_tile_map(p, b, 9 + TQ, shapes()[shape].rx, shapes()[shape].ry, map + b);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
+    static cudaError_t launch(const KParams &p, int shape, const CUtensorMap &map, int src, int k, cudaStream_t st) {
+        static const TileKernel<S> kernels[N] = {k_tile<S, TQ, BGK, RX, RY, T, MINB>...};
+        static std::atomic<bool> ready[N][kMaxDevices];
+        if (shape < 0 || shape >= N) return cudaErrorInvalidValue;
+        return launch_tile<S>(kernels[shape], shapes()[shape], ready[shape], p, map, src, k, st);
+    }
+    static const TileLaunchers *get() {
+        static const TileLaunchers L = {&plan, &maps, &launch};
+        return &L;
+    }
+};
+
+}  // namespace nomrt
