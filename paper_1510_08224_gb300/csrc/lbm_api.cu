@@ -479,11 +479,14 @@ bool plan_tiles(lbm_lattice *h) {
     return h->tile_plan.shape >= 0;
 }
 
-// n >= 2 steps as evenly sized launches of at most tile_plan.steps steps. Each is a
+// n >= 2 steps as evenly sized launches of at most tile_plan.steps steps, as many
+// launches as steps modulo 2: an even run ends on the buffer it began on, so that
+// a caller's graph of one can be replayed with other even runs between. Each is a
 // programmatic dependent of the one before and costs the GPU more time than its
 // launch costs the host, so they are launched directly.
 lbm_status step_tiles(lbm_lattice *h, int64_t n) {
-    const int64_t launches = (n + h->tile_plan.steps - 1) / h->tile_plan.steps;
+    int64_t launches = (n + h->tile_plan.steps - 1) / h->tile_plan.steps;
+    launches += (launches ^ n) & 1;
     for (int64_t i = launches; i > 0; --i) {
         const int k = (int)((n + i - 1) / i);
         cudaError_t e = h->tile->launch(h->kp, h->tile_plan.shape, h->tile_map[h->cur], h->cur, k, h->stream);

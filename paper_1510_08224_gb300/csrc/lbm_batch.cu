@@ -5,7 +5,7 @@
 //
 // Launch groups: up to kGroupLats members whose kinetic rates (s_e, s_q,
 // s_eps, zeta_e, zeta_nu, varpi) agree travel in one launch. Their
-// descriptors (buffers, geometry, and the eleven collision values that follow
+// descriptors (buffers, geometry, and the collision values that follow
 // from each member's own nu, alpha, g beta, T0 and body force) and the
 // group's shared rates form one __grid_constant__ kernel parameter. The
 // shared rates sit at fixed offsets of the parameter bank, so the collision
@@ -27,6 +27,10 @@
 // block of a 1-D grid; the persistent kernel's resident blocks take runs of
 // rows_per_unit consecutive virtual blocks, step after step.
 //
+// The FUSED kind with its default config takes several steps per launch where
+// every member can (tile_batch.cuh); single steps and the other configs run as
+// above.
+//
 // Ping-pong: member l reads buffer (s + flip_l) & 1 at batch step s, where
 // flip_l is fixed when the lattice joins, so lattices that joined at different
 // times step in lockstep.
@@ -42,40 +46,15 @@
 #include "lattice_impl.h"
 #include "nomrt_kernels.cuh"
 #include "nomrt_lbm.h"
+#include "tile_batch.cuh"
 
 namespace nomrt {
 
 constexpr int kBatchThreads = 128;
 constexpr int kBatchConfigs = 5;  // resident blocks asked of ptxas: 4 + config
 constexpr int kFusedConfigs = 2 * kBatchConfigs;  // FUSED: configs 5-9 are 0-4 with one row segment per warp
-constexpr int kGroupLats = 64;    // members per launch (the parameter block holds their descriptors)
 constexpr long long kBarrierBudgetCycles = 4000000000LL;  // ~2 s at 2 GHz
 constexpr int kDefaultPersistentSteps = 32;
-
-// The values of the MRT collision (collide_x) that follow from one lattice's nu,
-// alpha, g beta, T0 and body force; the rest of RatesC<float> that it reads is
-// shared by a launch group.
-struct MemberRates {
-    float s_nu4, om_nu4, h_nu2, nh_nu, om_a, z_a, hx, hFy0, hg_beta, T_ref;
-};
-
-inline MemberRates member_rates(const RatesC<float> &r) {
-    return MemberRates{r.s_nu4, r.om_nu4, r.h_nu2, r.nh_nu, r.om_a, r.z_a, r.hx, r.hFy0, r.hg_beta, r.T_ref};
-}
-
-__host__ __device__ __forceinline__ void apply_member(RatesC<float> &r, const MemberRates &v) {
-    r.s_nu4 = v.s_nu4;
-    r.ns_nu4 = -v.s_nu4;
-    r.om_nu4 = v.om_nu4;
-    r.h_nu2 = v.h_nu2;
-    r.nh_nu = v.nh_nu;
-    r.om_a = v.om_a;
-    r.z_a = v.z_a;
-    r.hx = v.hx;
-    r.hFy0 = v.hFy0;
-    r.hg_beta = v.hg_beta;
-    r.T_ref = v.T_ref;
-}
 
 // Whether two lattices' rates agree outside their member-specific values.
 inline bool same_shared_rates(RatesC<float> a, RatesC<float> b) {
@@ -457,6 +436,11 @@ struct lbm_batch {
     double *h_res = nullptr;
     size_t cap_res = 0;
     std::vector<nomrt::GroupParams> groups;  // launch parameters, kGroupLats members each
+    // FUSED, default config: several steps per launch where every member can (shape -1: not). One launch
+    // descriptor per group and batch-step parity, tiles[2 g + parity]
+    nomrt::TilePlan tile_plan{-1, 0};
+    std::vector<nomrt::TileGroup> tiles;
+    std::vector<size_t> member_of;  // member index of slot m of group g, at g kGroupLats + m
     int64_t cells = 0;
     int nunits = 0;  // (row chunk, segment) virtual blocks per step
     bool dirty = true;
@@ -504,6 +488,55 @@ void drop_graph(lbm_batch *b) {
     }
 }
 
+// The several-steps-per-launch plan and descriptors of the launch groups.
+void plan_tiles(lbm_batch *b) {
+    b->tile_plan = nomrt::TilePlan{-1, 0};
+    b->tiles.clear();
+    const nomrt::TileBatchLaunchers *L = nomrt::tile_batch_launchers(b->storage);
+    std::vector<const nomrt::KParams *> kp;
+    for (const lbm_lattice *h : b->members) kp.push_back(&h->kp);
+    int dev = 0, sms = 0;
+    if (kp.empty() || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return;
+    nomrt::TilePlan plan = L->plan(kp.data(), (int)kp.size(), sms);
+    if (plan.shape < 0) return;
+    b->tiles.resize(2 * b->groups.size());
+    for (size_t gi = 0; gi < b->groups.size(); ++gi) {
+        const nomrt::GroupParams &G = b->groups[gi];
+        for (int parity = 0; parity < 2; ++parity) {
+            nomrt::TileGroup &t = b->tiles[2 * gi + parity];
+            std::memset(&t, 0, sizeof t);
+            t.rc = G.rc;
+            t.nlats = G.nlats;
+            t.status = b->d_status;
+        }
+        for (int m = 0; m < G.nlats; ++m) {
+            const lbm_lattice *h = b->members[b->member_of[gi * nomrt::kGroupLats + m]];
+            CUtensorMap maps[2];
+            std::memset(maps, 0, sizeof maps);
+            if (L->maps(h->kp, plan.shape, maps) != cudaSuccess) {
+                cudaGetLastError();
+                b->tiles.clear();
+                return;
+            }
+            for (int parity = 0; parity < 2; ++parity) {
+                nomrt::TileMember &t = b->tiles[2 * gi + parity].lat[m];
+                const int sel = (parity + G.lat[m].flip) & 1;
+                t.map = maps[sel];
+                t.g = G.lat[m].g;
+                t.src = h->kp.pop[sel];
+                t.dst = h->kp.pop[1 - sel];
+                t.plane = h->kp.plane;
+                t.v = G.lat[m].v;
+                t.walls = nomrt::TileWalls{h->kp.n_walls, h->kp.moving};
+                t.row0 = h->kp.py ? 0 : 1;
+            }
+        }
+    }
+    b->tile_plan = plan;
+}
+
 // Rebuild the launch groups after a membership or shape change: members join
 // the first group whose shared rates equal theirs and that has room.
 lbm_status rebuild(lbm_batch *b) {
@@ -511,6 +544,7 @@ lbm_status rebuild(lbm_batch *b) {
     drop_graph(b);
     b->cells = 0;
     b->groups.clear();
+    b->member_of.clear();
     for (size_t l = 0; l < b->members.size(); ++l) {
         lbm_lattice *h = b->members[l];
         const nomrt::KParams &kp = h->kp;
@@ -528,6 +562,8 @@ lbm_status rebuild(lbm_batch *b) {
             std::memset(G, 0, sizeof(nomrt::GroupParams));
             G->rc = r;
         }
+        b->member_of.resize(b->groups.size() * nomrt::kGroupLats);
+        b->member_of[(size_t)(G - b->groups.data()) * nomrt::kGroupLats + G->nlats] = l;
         nomrt::GridLat &gl = G->lat[G->nlats];
         gl.g = nomrt::make_geom(kp);
         const size_t eb = h->storage == LBM_F16_SHIFTED ? 2 : 4;
@@ -579,6 +615,7 @@ lbm_status rebuild(lbm_batch *b) {
         at += (size_t)G.nvb;
         b->nunits += G.nvb;
     }
+    plan_tiles(b);
     b->dirty = false;
     return LBM_OK;
 }
@@ -685,8 +722,31 @@ cudaError_t launch_persistent_steps(lbm_batch *b, int config, int parity, int k,
     return cudaSuccess;
 }
 
+// k steps of every member in one launch per group.
+cudaError_t launch_tile_steps(lbm_batch *b, int parity, int k, cudaStream_t st) {
+    const nomrt::TileBatchLaunchers *L = nomrt::tile_batch_launchers(b->storage);
+    for (size_t gi = 0; gi < b->groups.size(); ++gi) {
+        cudaError_t e = L->launch(b->tiles[2 * gi + parity], b->tile_plan.shape, k, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_steps(lbm_batch *b, int parity, int n, cudaStream_t st) {
     if (b->kind == LBM_BATCH_CONCURRENT) return launch_concurrent(b, n, st, true);
+    if (b->kind == LBM_BATCH_FUSED && b->config < 0 && b->tile_plan.shape >= 0 && n > 1) {
+        // as many launches as steps modulo 2, so that the buffers' parity stays that of the steps
+        int launches = (n + b->tile_plan.steps - 1) / b->tile_plan.steps;
+        launches += (launches ^ n) & 1;
+        for (int i = launches; i > 0; --i) {
+            const int k = (n + i - 1) / i;
+            cudaError_t e = launch_tile_steps(b, parity, k, st);
+            if (e != cudaSuccess) return e;
+            parity ^= 1;
+            n -= k;
+        }
+        return cudaSuccess;
+    }
     // members with NEE walls need their boundary-node pass between steps: one launch per step
     if (b->kind == LBM_BATCH_PERSISTENT && !any_nee(b)) {
         while (n > 0) {
@@ -900,7 +960,7 @@ lbm_status lbm_batch_sync(lbm_batch *b) {
         const int zero = 0;
         cudaMemcpy(b->d_status, &zero, sizeof zero, cudaMemcpyHostToDevice);
         cudaMemset(b->d_bar, 0, 4 * sizeof(unsigned));
-        return bfail(b, LBM_ETIMEOUT, "the persistent batch kernel gave up a grid barrier");
+        return bfail(b, LBM_ETIMEOUT, "a batch kernel gave up a bounded wait (a grid barrier or a copy)");
     }
     if constexpr (nomrt::kBoundsBuild) {
         // the members' bounds words (the word after each lattice's status word)
@@ -1008,6 +1068,22 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *best_kind,
     }
     b->member_variant = own_variant;
     b->member_config = own_config;
+    // the default config's several steps per launch: a launch reads the current buffers and writes the others
+    float tile_ms = INFINITY;
+    if (b->tile_plan.shape >= 0 && out == LBM_OK) {
+        const int per = b->tile_plan.steps;
+        cudaError_t e = timed(
+            [&](int n) -> cudaError_t {
+                for (int done = 0; done < n; done += per) {
+                    cudaError_t le = launch_tile_steps(b, parity, per, b->stream);
+                    if (le != cudaSuccess) return le;
+                }
+                return cudaSuccess;
+            },
+            1, &tile_ms);
+        if (e != cudaSuccess) out = bcuda(b, e, "tuning launch (several steps)");
+        else tile_ms *= (float)trial_steps / (float)((trial_steps + per - 1) / per * per);
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (out != LBM_OK) return out;
@@ -1015,7 +1091,10 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *best_kind,
     int best = 0;
     for (int c = 1; c < kCand; ++c)
         if (ms[c] < ms[best]) best = c;
-    if (best < kPers) {
+    if (tile_ms < ms[best]) {
+        b->kind = LBM_BATCH_FUSED;
+        b->config = -1;
+    } else if (best < kPers) {
         b->kind = LBM_BATCH_FUSED;
         b->config = best;
     } else if (best < kConc) {
@@ -1032,7 +1111,7 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *best_kind,
     }
     drop_graph(b);
     if (best_kind) *best_kind = b->kind;
-    if (best_config) *best_config = b->kind == LBM_BATCH_CONCURRENT ? best - kConc - 1 : b->config;
+    if (best_config) *best_config = b->kind == LBM_BATCH_CONCURRENT ? best - kConc - 1 : b->cfg();
     if (ms_per_step)
         for (int c = 0; c < kCand; ++c) ms_per_step[c] = ms[c];
     return LBM_OK;

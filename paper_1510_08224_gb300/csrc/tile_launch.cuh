@@ -65,21 +65,35 @@ constexpr double kL2Bytes = 100e6;          // what of the 129 MB L2 two buffers
 // launch; so do FP16 lattices whose single steps are bound by HBM (1024^2 cells:
 // 14.0 us a step against 17.4; 600^2: 9.1 against 7.9), where the FP32 images a
 // block keeps cost more than the passes over memory they save.
-inline TilePlan choose_tile(const KParams &p, int nq, int elem, const TileShape *shapes, int n_shapes, int sms) {
+inline TilePlan choose_tile(const KParams *const *lats, int n, int nq, int elem, const TileShape *shapes,
+                            int n_shapes, int sms) {
     TilePlan best{-1, 0};
-    double least = 0;
-    const TileCover c = tile_cover(p);
-    if (p.n_nee > 0 || p.n_walls > kTileWalls || c.rows <= 0 || c.cols <= 0 || sms <= 0) return best;
-    if (elem == 2 && (long long)p.nx * p.ny > kTileMostF16) return best;
+    double least = 0, cells = 0;
+    if (n < 1 || sms <= 0) return best;
+    for (int m = 0; m < n; ++m) {
+        const KParams &p = *lats[m];
+        const TileCover c = tile_cover(p);
+        if (p.n_nee > 0 || p.n_walls > kTileWalls || (n == 1 && (c.rows <= 0 || c.cols <= 0))) return best;
+        cells += (double)p.nx * p.ny;
+    }
+    if (elem == 2 && cells > kTileMostF16) return best;
     const double cell_bytes = 2.0 * nq * elem;
-    const bool fits_l2 = cell_bytes * p.nx * p.ny < kL2Bytes;
+    const bool fits_l2 = cell_bytes * cells < kL2Bytes;
     for (int i = 0; i < n_shapes; ++i)
         for (int k = 2; k <= kTileMaxSteps; ++k) {
             const int tx = shape_cols(shapes[i], k), ty = shape_rows(shapes[i], k);
             if (tx < 4 || ty < 2) break;
-            const long long gx = (c.cols + tx - 1) / tx, gy = (c.rows + ty - 1) / ty;
-            if (gy > 65535 || gx * gy > 0x3FFFFFFF) continue;  // the launch grid's y limit
-            const double t = tile_cycles(shapes[i], k, gx * gy, cell_bytes, fits_l2, sms) / k;
+            long long tiles = 0;
+            bool fits = true;
+            for (int m = 0; m < n; ++m) {
+                const TileCover c = tile_cover(*lats[m]);
+                if (c.rows <= 0 || c.cols <= 0) continue;
+                const long long gx = (c.cols + tx - 1) / tx, gy = (c.rows + ty - 1) / ty;
+                fits = fits && (n > 1 || gy <= 65535);  // a lattice alone: the launch grid's y limit
+                tiles += gx * gy;
+            }
+            if (!fits || tiles > 0x3FFFFFFF) continue;
+            const double t = tile_cycles(shapes[i], k, tiles, cell_bytes, fits_l2, sms) / k;
             if (best.shape < 0 || t < least) {
                 best = TilePlan{i, k};
                 least = t;
@@ -144,19 +158,27 @@ template <typename S>
 using TileKernel = void (*)(const Planes<S>, const Geom, const RatesC<float>, const CUtensorMap, TileWalls, int, int,
                             int, int, int *);
 
+// The current device, the kernel's shared-memory limit raised on it once.
+template <typename K>
+cudaError_t tile_ready(K kern, std::atomic<bool> *ready, int *dev) {
+    cudaError_t e = cudaGetDevice(dev);
+    if (e != cudaSuccess) return e;
+    if (*dev < 0 || *dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    if (!ready[*dev].load(std::memory_order_acquire)) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return e;
+        ready[*dev].store(true, std::memory_order_release);
+    }
+    return cudaSuccess;
+}
+
 // One launch of k steps.
 template <typename S>
 cudaError_t launch_tile(TileKernel<S> kern, const TileShape &s, std::atomic<bool> *ready, const KParams &p,
                         const CUtensorMap &map, int src, int k, cudaStream_t st) {
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = tile_ready(kern, ready, &dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (!ready[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        if (e != cudaSuccess) return e;
-        ready[dev].store(true, std::memory_order_release);
-    }
     const int sms = tile_sms(dev);
     const TileCover c = tile_cover(p);
     const int tx = shape_cols(s, k), ty = shape_rows(s, k);
@@ -194,7 +216,10 @@ struct TileSet<S, TQ, BGK, ShapeOf<RX, RY, T, MINB>...> {
         static const TileShape s[N] = {TileShape{RX, RY, T, MINB, TileLayout<TQ, RX, RY>::bytes()}...};
         return s;
     }
-    static TilePlan plan(const KParams &p, int sms) { return choose_tile(p, 9 + TQ, (int)sizeof(S), shapes(), N, sms); }
+    static TilePlan plan(const KParams &p, int sms) {
+        const KParams *const one = &p;
+        return choose_tile(&one, 1, 9 + TQ, (int)sizeof(S), shapes(), N, sms);
+    }
     static cudaError_t maps(const KParams &p, int shape, CUtensorMap map[2]) {
         if (shape < 0 || shape >= N) return cudaErrorInvalidValue;
         if (sizeof(S) != 4) return cudaSuccess;  // FP16 regions are not copied through a tensor map

@@ -73,7 +73,8 @@ def test_runs_equal_single_steps(name, model, storage):
 
 
 def test_runs_inside_a_callers_capture():
-    """Runs of several steps recorded into a caller's CUDA graph and replayed."""
+    """An even run recorded into a caller's CUDA graph and replayed, other even
+    runs between the replays."""
     import torch
     import paper_1510_08224_gb300 as P
     case = CASES["cavity_65x64"]
@@ -82,10 +83,11 @@ def test_runs_inside_a_callers_capture():
         a, b = P.Lattice(case, storage="f32", stream=side), P.Lattice(case, storage="f32", stream=side)
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph, stream=side):
-            a.step(16)  # two launches: the graph starts and ends on the same buffer
-        for _ in range(3):
+            a.step(8)
+        for n in (2, 20, 8):
             graph.replay()
-        b.step(48)
+            a.step(n)
+            b.step(8 + n)
     side.synchronize()
     for u, v in zip(a.populations(), b.populations()):
         assert np.array_equal(u, v)
