@@ -2,6 +2,7 @@
 // Included once per kernel translation unit.
 #pragma once
 
+#include <algorithm>
 #include <atomic>
 
 #include "nomrt_kernels.cuh"
@@ -119,40 +120,6 @@ cudaError_t launch_nee(const KParams &p, int src, cudaStream_t st) {
 template <typename S>
 cudaError_t launch_step_main(const KParams &p, int src, cudaStream_t st);
 
-// One step: the main kernel over fluid cells, then the boundary nodes of NEE walls.
-template <typename S>
-cudaError_t launch_step(const KParams &p, int src, cudaStream_t st) {
-    cudaError_t e = launch_step_main<S>(p, src, st);
-    if (e != cudaSuccess) return e;
-    return launch_nee<S>(p, src, st);
-}
-
-template <typename S>
-cudaError_t launch_step_main(const KParams &p, int src, cudaStream_t st) {
-    int variant = p.variant;
-    KParams q = p;
-    if constexpr (Store<S>::kShifted) {
-        // fastest measured on GB300 (4096 x 2048 cells): four cells per thread
-        if (variant == kStepAuto) {
-            variant = kStepVec4;
-            // VEC4 configs measured fastest on GB300 (4096 x 2048 cells, with the L2
-            // prefetch of the link map): D2Q5 5 resident blocks per SM (4 for BGK in FP32);
-            // the D2Q9 temperature model, which keeps nine more values per cell in
-            // registers, 4
-            if (p.tq == 9) q.config = 0;
-            else q.config = (p.bgk && sizeof(S) == 4) ? 0 : 1;
-            // FP32 MRT D2Q5 rows that are not a multiple of 512 cells: the per-warp form,
-            // which leaves no warp of a block idle at a row's end (600 x 600: 0.77 -> 0.82
-            // of the copy peak, 1100 x 900: 0.88 -> 0.91); in FP16 its per-warp prefetches
-            // measured slower (4096 x 2048: 0.78 against 0.96)
-            if (sizeof(S) == 4 && p.tq == 5 && !p.bgk && p.pitch % 512 != 0) variant = kStepVec4w;
-        }
-    } else {
-        variant = kStepScalar;
-    }
-    return launch_step_variant<S>(q, variant, src, st);
-}
-
 // SMs of the current device, read once per device (0 if it cannot be read).
 inline int device_sms() {
     constexpr int kDevices = 16;
@@ -163,6 +130,67 @@ inline int device_sms() {
     if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
         sms[dev].store(n, std::memory_order_relaxed);
     return n;
+}
+
+constexpr int kStep64Wave = 40;  // blocks per SM in about four waves of k_step64
+
+// One FP64 step, boundary nodes included.
+template <int TQ, bool BGK>
+cudaError_t launch_step64(const KParams &p, int src, cudaStream_t st) {
+    const int row0 = p.py ? 0 : 1;  // the first and last row of a non-periodic y hold no fluid cell
+    const long long cells = (long long)std::max(0, p.ny - 2 * row0) * p.nx;
+    const int node_blocks = (p.n_nee + kStep64Threads - 1) / kStep64Threads;
+    const long long blocks = node_blocks + (cells + kStep64Threads - 1) / kStep64Threads;
+    if (blocks == 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kStep64Threads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    // a dependent only where its grid spans several waves: the blocks of a smaller one would settle where
+    // the previous step's blocks end first, and leave the SMs unevenly loaded (256^2 cells: 30 us a step)
+    const bool dependent = blocks > (long long)device_sms() * kStep64Wave;
+    cfg.attrs = dependent ? attr : nullptr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_step64<TQ, BGK>, make_planes<double>(p, src), make_geom(p),
+                              make_rates<double>(p), p.nee, p.n_nee, node_blocks, row0, (int)cells);
+}
+
+// One step: the main kernel over fluid cells, then the boundary nodes of NEE walls.
+template <typename S>
+cudaError_t launch_step(const KParams &p, int src, cudaStream_t st) {
+    if constexpr (sizeof(S) == 8) {
+        if (p.tq == 9) return p.bgk ? launch_step64<9, true>(p, src, st) : launch_step64<9, false>(p, src, st);
+        return p.bgk ? launch_step64<5, true>(p, src, st) : launch_step64<5, false>(p, src, st);
+    } else {
+        cudaError_t e = launch_step_main<S>(p, src, st);
+        if (e != cudaSuccess) return e;
+        return launch_nee<S>(p, src, st);
+    }
+}
+
+template <typename S>
+cudaError_t launch_step_main(const KParams &p, int src, cudaStream_t st) {
+    int variant = p.variant;
+    KParams q = p;
+    // fastest measured on GB300 (4096 x 2048 cells): four cells per thread
+    if (variant == kStepAuto) {
+        variant = kStepVec4;
+        // VEC4 configs measured fastest on GB300 (4096 x 2048 cells, with the L2
+        // prefetch of the link map): D2Q5 5 resident blocks per SM (4 for BGK in FP32);
+        // the D2Q9 temperature model, which keeps nine more values per cell in
+        // registers, 4
+        if (p.tq == 9) q.config = 0;
+        else q.config = (p.bgk && sizeof(S) == 4) ? 0 : 1;
+        // FP32 MRT D2Q5 rows that are not a multiple of 512 cells: the per-warp form,
+        // which leaves no warp of a block idle at a row's end (600 x 600: 0.77 -> 0.82
+        // of the copy peak, 1100 x 900: 0.88 -> 0.91); in FP16 its per-warp prefetches
+        // measured slower (4096 x 2048: 0.78 against 0.96)
+        if (sizeof(S) == 4 && p.tq == 5 && !p.bgk && p.pitch % 512 != 0) variant = kStepVec4w;
+    }
+    return launch_step_variant<S>(q, variant, src, st);
 }
 
 // A step of the four-cell kernel, as a programmatic dependent of the launch before
@@ -340,7 +368,8 @@ template <typename S>
 Launchers make_launchers() {
     Launchers L;
     L.step = &launch_step<S>;
-    L.nee = &launch_nee<S>;
+    L.nee = nullptr;  // FP64 steps take the nodes along
+    if constexpr (Store<S>::kShifted) L.nee = &launch_nee<S>;
     L.init_rows = &launch_init_rows<S>;
     L.macro_rows = &launch_macro_rows<S>;
     L.export_rows = &launch_export_rows<S>;

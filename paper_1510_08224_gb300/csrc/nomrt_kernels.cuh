@@ -98,6 +98,9 @@ struct RatesC {
     C h_e, h_nu2, nh_nu, h3eps;   // 1 - s_e/2, (1 - s_nu/2)/2, -(1 - s_nu/2), (1 - s_eps/2)/3
     C om_ze4, zv_e4, om_zn4;
     C hx, hFy0, hg_beta;          // ax / 2, Fy0 / 2, g_beta / 2
+    // products of the above that the FP64 collision takes ready-made (collide_d): h_nu ax / 2, ax / 12,
+    // s_e / 6, s_q / 12, s_eps / 36, s_eps / 12, zeta_alpha / 2, zeta_alpha T_ref / 2, (1 - zeta_alpha) / 2
+    C hnu_hx, hx6, s_e6, s_q12, s_eps36, s_eps12, z_a2, z_aT2, om_a2;
     C varpi;                      // Eq. 28
     // D2Q9 temperature model (Eqs. 31-33): zeta_e, zeta_nu, zeta_q, zeta_eps and theta
     C z_e, z_nu, om_zq, z_q, om_zeps, z_eps, theta;
@@ -138,6 +141,19 @@ inline RatesC<C> make_rates(const KParams &p) {
     r.hx = h * r.ax;
     r.hFy0 = h * r.Fy0;
     r.hg_beta = h * r.g_beta;
+    if (sizeof(C) == 8) {
+        r.hnu_hx = r.h_nu * r.hx;
+        r.hx6 = r.hx / (C)6;
+        r.s_e6 = r.s_e4 * (C)2 / (C)3;
+        r.s_q12 = r.s_q2 / (C)6;
+        r.s_eps36 = r.s_eps4 / (C)9;
+        r.s_eps12 = r.s_eps4 / (C)3;
+        r.z_a2 = h * r.z_a;
+        r.z_aT2 = r.z_a2 * r.T_ref;
+        r.om_a2 = h * r.om_a;
+    } else {
+        r.hnu_hx = r.hx6 = r.s_e6 = r.s_q12 = r.s_eps36 = r.s_eps12 = r.z_a2 = r.z_aT2 = r.om_a2 = (C)0;
+    }
     r.varpi = (C)p.varpi;
     r.z_e = (C)p.z_e;
     r.z_nu = (C)p.z_nu;
@@ -344,6 +360,31 @@ __device__ __forceinline__ void nee_rebuild(const S *const *src, const Geom &g,
     const C uwx = (C)w->uwx, uwy = (C)w->uwy;
     const C Tf = r.T_ref + M.dT;
     const C Tb = w->adiabatic != 0.0 ? Tf : (C)w->Tw;
+    if constexpr (sizeof(C) == 8 && TQ == 5) {
+        // FP64: the differences of the equilibria through s = u_w + u_f and d = u_w - u_f,
+        //   f_i += w_i [e.d (3 + 4.5 e.s) - 1.5 s.d],  g_i += varpi/4 (T_b - T_f) + e.(u_w T_b - u_f T_f)/2,
+        // opposite directions together: about 45 FP64 operations instead of 140
+        const C sx = uwx + M.ux, sy = uwy + M.uy, dx = uwx - M.ux, dy = uwy - M.uy;
+        const C iso = C(-1.5) * (sx * dx + sy * dy);
+        auto pair = [&](int i, int j, C w, C es, C ed) {
+            const C even = w * (iso + C(4.5) * (es * ed)), odd = (C(3) * w) * ed;
+            f[i] += even + odd;
+            f[j] += even - odd;
+        };
+        f[0] += C(4.0 / 9) * iso;
+        pair(1, 3, C(1.0 / 9), sx, dx);
+        pair(2, 4, C(1.0 / 9), sy, dy);
+        pair(5, 7, C(1.0 / 36), sx + sy, dx + dy);
+        pair(6, 8, C(1.0 / 36), sy - sx, dy - dx);
+        const C dT = Tb - Tf, q = C(0.25) * r.varpi * dT;
+        const C gx = C(0.5) * (uwx * Tb - M.ux * Tf), gy = C(0.5) * (uwy * Tb - M.uy * Tf);
+        t[0] += (C(1) - r.varpi) * dT;
+        t[1] += q + gx;
+        t[3] += q - gx;
+        t[2] += q + gy;
+        t[4] += q - gy;
+        return;
+    }
     const C uf2 = M.ux * M.ux + M.uy * M.uy, uw2 = uwx * uwx + uwy * uwy;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -565,6 +606,72 @@ __device__ __forceinline__ void collide_x(const R &r, T f[9], T t[TQ]) {
     }
 }
 
+// The MRT collision with the D2Q5 temperature lattice in FP64: collide_x's
+// moments with the products regrouped for the fewest operations, 94 instead of
+// 101 (FP64 steps are bound by that pipe: two lanes per cycle and SM). The terms
+// of p4 and p5 share a = s_nu/4 u_x + h_nu F_x/2 and b likewise in y:
+//   p4 = (1 - s_nu)/4 m4 + u_x a - u_y b,  p5 = (1 - s_nu)/4 m5 + (u_x b + u_y a)/2;
+// p3, p8, p6 and p7 take their moments with ready-made coefficients, and the
+// temperature fluxes z_a T/2 at once.
+__device__ __forceinline__ void collide_d(const RatesC<double> &r, double f[9], double t[5]) {
+    const double n0 = ((t[0] + t[1]) + (t[2] + t[3])) + t[4];  // T - T_ref
+    const double hFx = r.hx;
+    const double hFy = __fma_rn(r.hg_beta, n0, r.hFy0);  // F / 2 (Eq. 4)
+    // D2Q9 forward map (Eq. 13)
+    const double a13 = f[1] + f[3], d13 = f[1] - f[3];
+    const double a24 = f[2] + f[4], d24 = f[2] - f[4];
+    const double a57 = f[5] + f[7], d57 = f[5] - f[7];
+    const double a68 = f[6] + f[8], d68 = f[6] - f[8];
+    const double D = a57 + a68, A4 = a13 + a24;
+    const double m0 = (f[0] + A4) + D;
+    const double m6 = d57 + d68, m7 = d57 - d68;
+    const double jx = d13 + m7, jy = d24 + m6;
+    const double m3 = __fma_rn(2.0, D, A4);
+    const double m4 = a13 - a24, m5 = a57 - a68;
+    // Eq. 19 with rho0 = 1
+    const double ux = jx + hFx, uy = jy + hFy;
+    const double uu = __fma_rn(ux, ux, __dmul_rn(uy, uy));
+    const double uF = __fma_rn(ux, hFx, __dmul_rn(uy, hFy));  // u.F / 2
+    // Eq. 8; p1, p2 halved, p3..p8 quartered
+    const double a = __fma_rn(r.s_nu4, ux, r.hnu_hx), b = __fma_rn(r.s_nu4, uy, __dmul_rn(r.h_nu, hFy));
+    const double p1 = __fma_rn(0.5, jx, hFx);
+    const double p2 = __fma_rn(0.5, jy, hFy);
+    const double p3 = __fma_rn(r.om_e4, m3, __fma_rn(r.s_e6, m0, __fma_rn(r.s_e4, uu, __dmul_rn(r.h_e, uF))));
+    const double p4 = __fma_rn(ux, a, __fma_rn(-uy, b, __dmul_rn(r.om_nu4, m4)));
+    const double p5 = __fma_rn(0.5, __fma_rn(ux, b, __dmul_rn(uy, a)), __dmul_rn(r.om_nu4, m5));
+    const double p6 = __fma_rn(r.om_q4, m6, __fma_rn(r.s_q12, jy, __dmul_rn(1.0 / 6.0, hFy)));
+    const double p7 = __fma_rn(r.om_q4, m7, __fma_rn(r.s_q12, jx, r.hx6));
+    const double p8 = __fma_rn(r.om_eps4, D, __fma_rn(r.s_eps36, m0, __fma_rn(r.s_eps12, uu, __dmul_rn(r.h3eps, uF))));
+    // back map (Eq. A1)
+    const double A = __fma_rn(-2.0, p8, p3);
+    const double h1 = __fma_rn(-2.0, p7, p1), h2 = __fma_rn(-2.0, p6, p2);
+    const double P = p8 + p5, Q = p6 + p7, Rm = p8 - p5, Sx = p6 - p7;
+    const double AB = A + p4, AmB = A - p4;
+    f[0] = __fma_rn(4.0, p8, __fma_rn(-4.0, p3, m0));
+    f[1] = AB + h1;
+    f[3] = AB - h1;
+    f[2] = AmB + h2;
+    f[4] = AmB - h2;
+    f[5] = P + Q;
+    f[7] = P - Q;
+    f[6] = Rm + Sx;
+    f[8] = Rm - Sx;
+    // D2Q5 forward map (Eq. 26), relaxation (Eq. 24; q1, q2 halved, q3, q4 quartered) and back map (Eq. A2)
+    const double s13 = t[1] + t[3], s24 = t[2] + t[4];
+    const double n1 = t[1] - t[3], n2 = t[2] - t[4];
+    const double n3 = s13 + s24, n4 = s13 - s24;
+    const double zT = __fma_rn(r.z_a2, n0, r.z_aT2);
+    const double q1 = __fma_rn(ux, zT, __dmul_rn(r.om_a2, n1));
+    const double q2 = __fma_rn(uy, zT, __dmul_rn(r.om_a2, n2));
+    const double q3 = __fma_rn(r.om_ze4, n3, __dmul_rn(r.zv_e4, n0));
+    const double c34 = __fma_rn(r.om_zn4, n4, q3), c3m4 = __fma_rn(-r.om_zn4, n4, q3);
+    t[0] = __fma_rn(-4.0, q3, n0);
+    t[1] = c34 + q1;
+    t[3] = c34 - q1;
+    t[2] = c3m4 + q2;
+    t[4] = c3m4 - q2;
+}
+
 // ------------------------------------------------------------ BGK collision
 
 // e_I . (x, y) for the D2Q9 velocities of Eq. 5 (I >= 1), exactly.
@@ -672,6 +779,7 @@ __device__ __forceinline__ void collide_cell(const RatesC<typename Store<S>::C> 
                                              typename Store<S>::C t[TQ]) {
     using C = typename Store<S>::C;
     if constexpr (BGK) collide_bgk_x<C, RatesC<C>, TQ>(r, f, t);
+    else if constexpr (sizeof(C) == 8 && TQ == 5) collide_d(r, f, t);
     else collide_x<C, TQ>(r, f, t);
 }
 
@@ -783,6 +891,54 @@ __global__ void __launch_bounds__(128) k_nee(const Planes<S> pl, const Geom g, c
 #pragma unroll
     for (int q = 0; q < TQ; ++q)
         if (NOMRT_OK(g, pl.dst[9 + q] + off, sizeof(S), 27)) Store<S>::st(pl.dst[9 + q] + off, t[q]);
+}
+
+// The FP64 step: one cell per thread, cells numbered along the rows without
+// regard to their ends, in blocks of two warps; the boundary nodes of node-based
+// walls are the first node_blocks blocks' (they read the same source buffer and
+// write cells no other thread writes). Bound by the FP64 pipe: 94 instructions
+// of 16 cycles per warp and SM. Small blocks and no idle row ends because a
+// lattice of 256^2 cells gives an SM about 14 warps: with 128 x 2 blocks (three
+// per row pair, the third nearly empty) some SMs ran half as many again, and a
+// second launch for the nodes, 16 warps on 4 SMs, took as long as the cells.
+// Measured, us per step, before -> now: 256^2 26.1 -> 15.4, 128^2 10.2 -> 6.6,
+// node-based walls 256^2 39.6 -> 15.7 and 128^2 23.8 -> 8.6, 1000^2 218 -> 182
+// (5.5e9 cells/s: the pipe's measured rate).
+constexpr int kStep64Threads = 64;
+
+template <int TQ, bool BGK>
+__global__ void __launch_bounds__(kStep64Threads)
+    k_step64(const Planes<double> pl, const Geom g, const RatesC<double> r, const int2 *nee, int n_nee,
+             int node_blocks, int row0, int cells) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    double f[9], t[TQ];
+    int off;
+    if ((int)blockIdx.x < node_blocks) {
+        const int i = (int)(blockIdx.x * kStep64Threads + threadIdx.x);
+        if (i >= n_nee || !NOMRT_OK(g, nee + i, sizeof(int2), 25)) return;
+        const int2 e = nee[i];
+        off = e.x;
+        const int d = e.y & 0xFF, k = e.y >> 8;
+        const int y = off / g.pitch, x = off - y * g.pitch;
+        if (!NOMRT_OK(g, g.walls + k, sizeof(WallDev), 26)) return;
+        nee_rebuild<double, TQ>(pl.src, g, r, x, y, d, g.walls + k, f, t);
+    } else {
+        const int i = (int)((blockIdx.x - node_blocks) * kStep64Threads + threadIdx.x);
+        if (i >= cells) return;
+        const int row = i / g.nx, x = i - row * g.nx, y = row0 + row;
+        off = y * g.pitch + x;
+        const unsigned m = NOMRT_OK(g, g.mask + off, 1, 6) ? __ldg(g.mask + off) : (unsigned)kSolid;
+        if (m == kSolid) return;
+        pull<double, TQ>(pl.src, g, x, y, m, f, t);
+    }
+    collide_cell<double, TQ, BGK>(r, f, t);
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+        if (NOMRT_OK(g, pl.dst[q] + off, sizeof(double), 7)) pl.dst[q][off] = f[q];
+#pragma unroll
+    for (int q = 0; q < TQ; ++q)
+        if (NOMRT_OK(g, pl.dst[9 + q] + off, sizeof(double), 7)) pl.dst[9 + q][off] = t[q];
 }
 
 // Initial state (rest equilibrium, Eqs. 22, 30 at u = 0) in the storage frame.

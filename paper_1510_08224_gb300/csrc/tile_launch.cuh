@@ -34,12 +34,14 @@ inline TileCover tile_cover(const KParams &p) {
 // its pipes, better the more of them are out of step with one another; and the
 // wave's bytes take their time on the way from and to HBM (or L2, for a lattice
 // that fits it), overlapped with the steps but not entirely. The constants are
-// a least-squares fit to 200 launches on lattices of 64^2 to 4096 x 2048 cells
-// with 2 to 8 steps per launch (rms error 12 %).
+// a least-squares fit to 551 timed launches of 16 shapes with 2 to 8 steps on
+// lattices of 64^2 to 4096 x 2048 cells and on batches of 24 to 64 cavities (rms
+// error 13 %); the shape and steps it picks run within 4 % of the fastest of
+// them on average, 19 % at worst (180^2).
 inline double tile_cycles(const TileShape &s, int k, long long tiles, double cell_bytes, bool fits_l2, int sms) {
-    constexpr double kLaunch = 9000, kBlock = 1770, kLatency = 1360, kRound = 0.7;
-    constexpr double kPairWarp[4] = {151, 110, 92, 91};  // cycles per 32 pairs with 1..4 blocks on the SM
-    constexpr double kHbm = 25.8, kL2 = 3 * kHbm;        // bytes per cycle and SM
+    constexpr double kLaunch = 12000, kBlock = 1570, kLatency = 612, kRound = 1.74;
+    constexpr double kPairWarp[4] = {137.5, 118.2, 107.7, 103.5};  // cycles per 32 pairs with 1..4 blocks on the SM
+    constexpr double kHbm = 40, kL2 = 3 * kHbm;                    // bytes per cycle and SM
     auto wave = [&](int n) {
         double steps = kBlock;
         for (int l = 1; l <= k; ++l) {
