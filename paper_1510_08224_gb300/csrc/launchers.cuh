@@ -132,30 +132,46 @@ inline int device_sms() {
     return n;
 }
 
-constexpr int kStep64Wave = 40;  // blocks per SM in about four waves of k_step64
+constexpr int kStep64Wave = 40;   // blocks per SM in about four waves of k_step64
+// Columns up to which a lattice of at most two rows per SM keeps the one-cell kernel's blocks of two rows:
+// one block of up to four warps with cells per SM (60 x 60, BGK: 5.5 against 5.8 us a step)
+constexpr int kStep64Narrow = 64;
+constexpr int kStep64ByRow = 4;   // warps per SM up to which its blocks lie along rows
 
 // One FP64 step, boundary nodes included.
 template <int TQ, bool BGK>
 cudaError_t launch_step64(const KParams &p, int src, cudaStream_t st) {
     const int row0 = p.py ? 0 : 1;  // the first and last row of a non-periodic y hold no fluid cell
-    const long long cells = (long long)std::max(0, p.ny - 2 * row0) * p.nx;
-    const int node_blocks = (p.n_nee + kStep64Threads - 1) / kStep64Threads;
-    const long long blocks = node_blocks + (cells + kStep64Threads - 1) / kStep64Threads;
+    const int rows = std::max(0, p.ny - 2 * row0);
+    const long long cells = (long long)rows * p.nx;
+    const long long sms = device_sms();
+    if (p.n_nee == 0 && p.nx <= kStep64Narrow && (rows + 1) / 2 <= sms) {
+        const dim3 b = step_block();
+        const dim3 grid((p.nx + b.x - 1) / b.x, (p.ny + b.y - 1) / b.y);
+        k_step<double, TQ, BGK><<<grid, b, 0, st>>>(make_planes<double>(p, src), make_geom(p), make_rates<double>(p));
+        return cudaGetLastError();
+    }
+    constexpr int T = 64;
+    const bool flat = p.n_nee > 0 || (long long)((p.nx + 31) / 32) * rows > sms * kStep64ByRow;
+    const int node_blocks = (p.n_nee + T - 1) / T;
+    const long long blocks = node_blocks + (cells + T - 1) / T;
     if (blocks == 0) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(kStep64Threads);
+    cfg.gridDim = flat ? dim3((unsigned)blocks) : dim3((p.nx + T - 1) / T, rows);
+    cfg.blockDim = dim3(T);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     // a dependent only where its grid spans several waves: the blocks of a smaller one would settle where
     // the previous step's blocks end first, and leave the SMs unevenly loaded (256^2 cells: 30 us a step)
-    const bool dependent = blocks > (long long)device_sms() * kStep64Wave;
+    const bool dependent = blocks > sms * kStep64Wave;
     cfg.attrs = dependent ? attr : nullptr;
     cfg.numAttrs = dependent ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_step64<TQ, BGK>, make_planes<double>(p, src), make_geom(p),
-                              make_rates<double>(p), p.nee, p.n_nee, node_blocks, row0, (int)cells);
+    auto kern = dependent ? (p.n_nee > 0 ? k_step64<TQ, BGK, true, true> : k_step64<TQ, BGK, false, true>)
+                          : (p.n_nee > 0 ? k_step64<TQ, BGK, true, false> : k_step64<TQ, BGK, false, false>);
+    return cudaLaunchKernelEx(&cfg, kern, make_planes<double>(p, src), make_geom(p), make_rates<double>(p), p.nee,
+                              p.n_nee, node_blocks, row0, (int)cells, flat ? 1 : 0);
 }
 
 // One step: the main kernel over fluid cells, then the boundary nodes of NEE walls.

@@ -893,10 +893,10 @@ __global__ void __launch_bounds__(128) k_nee(const Planes<S> pl, const Geom g, c
         if (NOMRT_OK(g, pl.dst[9 + q] + off, sizeof(S), 27)) Store<S>::st(pl.dst[9 + q] + off, t[q]);
 }
 
-// The FP64 step: one cell per thread, cells numbered along the rows without
-// regard to their ends, in blocks of two warps; the boundary nodes of node-based
-// walls are the first node_blocks blocks' (they read the same source buffer and
-// write cells no other thread writes). Bound by the FP64 pipe: 94 instructions
+// The FP64 step: one cell per thread in blocks of two warps, cells numbered along
+// the rows without regard to their ends (flat) or, in lattices of a few warps per
+// SM, where a step is a chain of latencies, along one row per grid row. NODES: the boundary nodes of node-based walls are the first blocks'
+// (they read the same source buffer and write cells no other thread writes). Bound by the FP64 pipe: 94 instructions
 // of 16 cycles per warp and SM. Small blocks and no idle row ends because a
 // lattice of 256^2 cells gives an SM about 14 warps: with 128 x 2 blocks (three
 // per row pair, the third nearly empty) some SMs ran half as many again, and a
@@ -904,18 +904,20 @@ __global__ void __launch_bounds__(128) k_nee(const Planes<S> pl, const Geom g, c
 // Measured, us per step, before -> now: 256^2 26.1 -> 15.4, 128^2 10.2 -> 6.6,
 // node-based walls 256^2 39.6 -> 15.7 and 128^2 23.8 -> 8.6, 1000^2 218 -> 182
 // (5.5e9 cells/s: the pipe's measured rate).
-constexpr int kStep64Threads = 64;
-
-template <int TQ, bool BGK>
-__global__ void __launch_bounds__(kStep64Threads)
+// MANY: a grid of several waves, launched as a programmatic dependent of the step
+// before it.
+template <int TQ, bool BGK, bool NODES, bool MANY>
+__global__ void __launch_bounds__(64)
     k_step64(const Planes<double> pl, const Geom g, const RatesC<double> r, const int2 *nee, int n_nee,
-             int node_blocks, int row0, int cells) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+             int node_blocks, int row0, int cells, int flat) {
+    if constexpr (MANY) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
     double f[9], t[TQ];
     int off;
-    if ((int)blockIdx.x < node_blocks) {
-        const int i = (int)(blockIdx.x * kStep64Threads + threadIdx.x);
+    if (NODES && (int)blockIdx.x < node_blocks) {
+        const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
         if (i >= n_nee || !NOMRT_OK(g, nee + i, sizeof(int2), 25)) return;
         const int2 e = nee[i];
         off = e.x;
@@ -924,9 +926,16 @@ __global__ void __launch_bounds__(kStep64Threads)
         if (!NOMRT_OK(g, g.walls + k, sizeof(WallDev), 26)) return;
         nee_rebuild<double, TQ>(pl.src, g, r, x, y, d, g.walls + k, f, t);
     } else {
-        const int i = (int)((blockIdx.x - node_blocks) * kStep64Threads + threadIdx.x);
-        if (i >= cells) return;
-        const int row = i / g.nx, x = i - row * g.nx, y = row0 + row;
+        int x = (int)(blockIdx.x * blockDim.x + threadIdx.x), y = row0 + (int)blockIdx.y;
+        if (flat) {
+            const int i = x - (NODES ? node_blocks * (int)blockDim.x : 0);
+            if (i >= cells) return;
+            const int row = i / g.nx;
+            x = i - row * g.nx;
+            y = row0 + row;
+        } else if (x >= g.nx) {
+            return;
+        }
         off = y * g.pitch + x;
         const unsigned m = NOMRT_OK(g, g.mask + off, 1, 6) ? __ldg(g.mask + off) : (unsigned)kSolid;
         if (m == kSolid) return;
