@@ -28,34 +28,41 @@ inline TileCover tile_cover(const KParams &p) {
     return TileCover{p.py ? 0 : 1, p.py ? p.ny : p.ny - 2, p.px ? p.nx : p.nx - 1};
 }
 
-// Estimated cycles of one launch of k steps, all its tiles: a launch's own cost,
-// then waves of resident blocks. A block's steps take at least their latency
-// (one pass of a thread over its pairs, a barrier); the blocks of an SM share
-// its pipes, better the more of them are out of step with one another; and the
-// wave's bytes take their time on the way from and to HBM (or L2, for a lattice
-// that fits it), overlapped with the steps but not entirely. The constants are
-// a least-squares fit to 551 timed launches of 16 shapes with 2 to 8 steps on
-// lattices of 64^2 to 4096 x 2048 cells and on batches of 24 to 64 cavities (rms
-// error 13 %); the shape and steps it picks run within 4 % of the fastest of
-// them on average, 19 % at worst (180^2).
+// Estimated cycles of one launch of k steps, all its tiles. Up to two waves of
+// resident blocks: a launch's own cost, and per wave the steps, each at least
+// its latency (one pass of a thread over its pairs, a barrier) or what the SM's
+// blocks take of its pipes when they start together. Many waves: the blocks are
+// out of step with one another and with the copies, so the slower of the pipes
+// and the way to HBM (or L2, for a lattice that fits it) sets the pace. The
+// constants are a least-squares fit to 551 timed launches of 16 shapes with 2
+// to 8 steps on lattices of 64^2 to 4096 x 2048 cells and on batches of 24 to
+// 64 cavities (rms error 13 %); the shape and steps it picks run within 2 % of
+// the fastest of them but for 180^2 cells (19 %).
 inline double tile_cycles(const TileShape &s, int k, long long tiles, double cell_bytes, bool fits_l2, int sms) {
-    constexpr double kLaunch = 12000, kBlock = 1570, kLatency = 612, kRound = 1.74;
-    constexpr double kPairWarp[4] = {137.5, 118.2, 107.7, 103.5};  // cycles per 32 pairs with 1..4 blocks on the SM
-    constexpr double kHbm = 40, kL2 = 3 * kHbm;                    // bytes per cycle and SM
+    constexpr double kLaunch = 11600, kLatency = 920, kRound = 1.18;
+    constexpr double kTogether[4] = {153, 141, 142, 125};  // cycles per 32 pairs with 1..4 blocks on the SM
+    constexpr double kBlock = 3640, kPairWarp = 80.3, kWarpStep = 8.1, kHbm = 21.2;  // many waves; bytes per cycle and SM
+    double pair_warps = 0;
+    const int cols = shape_cols(s, k), rows = shape_rows(s, k);
+    auto pairs = [&](int l) { return (s.ry / 2 - l) * (l < k ? s.rx : cols); };
+    for (int l = 1; l <= k; ++l) pair_warps += (pairs(l) + 31) / 32;
     auto wave = [&](int n) {
-        double steps = kBlock;
+        double t = 0;
         for (int l = 1; l <= k; ++l) {
-            const int pairs = (s.ry / 2 - l) * (l < k ? s.rx : shape_cols(s, k));
-            const int rounds = (pairs + s.threads - 1) / s.threads;
-            steps += std::max(kLatency * (1 + kRound * (rounds - 1)),
-                              n * ((pairs + 31) / 32) * kPairWarp[std::min(n, 4) - 1]);
+            const int rounds = (pairs(l) + s.threads - 1) / s.threads;
+            t += std::max(kLatency * (1 + kRound * (rounds - 1)),
+                          n * ((pairs(l) + 31) / 32) * kTogether[std::min(n, 4) - 1]);
         }
-        const double bytes = n * shape_cols(s, k) * shape_rows(s, k) * cell_bytes / (fits_l2 ? kL2 : kHbm);
-        return std::cbrt(steps * steps * steps + bytes * bytes * bytes);
+        return t;
     };
     const long long slots = (long long)sms * s.per_sm;
     const long long full = tiles / slots, rest = tiles % slots;
-    return kLaunch + (double)full * wave(s.per_sm) + (rest ? wave((int)((rest + sms - 1) / sms)) : 0.0);
+    if (full <= 1)
+        return kLaunch + (double)full * wave(s.per_sm) + (rest ? wave((int)((rest + sms - 1) / sms)) : 0.0);
+    const double steps = kBlock + s.per_sm * (pair_warps * kPairWarp + k * (s.threads / 32) * kWarpStep);
+    const double bytes = s.per_sm * cols * rows * cell_bytes / (fits_l2 ? 3 * kHbm : kHbm);
+    return kLaunch + std::pow(std::pow(steps, 7.5) + std::pow(bytes, 7.5), 1 / 7.5) * ((double)tiles / (double)slots) +
+           0.5 * wave(s.per_sm);
 }
 
 constexpr int kTileMaxSteps = 8;
