@@ -64,7 +64,12 @@ struct lbm_lattice {
     nomrt::TilePlan tile_plan{-1, 0};
     bool tile_planned = false;
     CUtensorMap tile_map[2];
+    bool recorded = false;  // some run was recorded into a caller's graph
 
+    nomrt::ReadMsg msg;  // a read-out's sums and status words, written by the GPU where it reaches host memory
+
+    // the reductions' block counter: a word of the status slot, zero between launches
+    unsigned *counter() const { return reinterpret_cast<unsigned *>(mem + lay.off_status + 64); }
     double *stage() const { return reinterpret_cast<double *>(mem + lay.off_stage); }
     double *partials() const { return reinterpret_cast<double *>(mem + lay.off_part); }
     double *result() const { return reinterpret_cast<double *>(mem + lay.off_res); }

@@ -326,15 +326,16 @@ cudaError_t launch_init_rows(const KParams &p, int buf, int r0, int r1, const do
 }
 
 template <typename S>
-cudaError_t launch_macro_rows(const KParams &p, int buf, int r0, int r1, double *const out[4], cudaStream_t st) {
+cudaError_t launch_macro_rows(const KParams &p, int buf, int r0, int r1, double *const out[4], ReadMsg *msg,
+                              cudaStream_t st) {
     using C = typename Store<S>::C;
     const dim3 grid((p.nx + 127) / 128, r1 - r0);
     if (p.tq == 9)
         k_macro_rows<S, 9><<<grid, 128, 0, st>>>(make_planes<S>(p, buf), make_geom(p), make_rates<C>(p), r0, r1,
-                                                 p.rho_ref, p.T_ref, out[0], out[1], out[2], out[3]);
+                                                 p.rho_ref, p.T_ref, out[0], out[1], out[2], out[3], msg, p.status);
     else
         k_macro_rows<S, 5><<<grid, 128, 0, st>>>(make_planes<S>(p, buf), make_geom(p), make_rates<C>(p), r0, r1,
-                                                 p.rho_ref, p.T_ref, out[0], out[1], out[2], out[3]);
+                                                 p.rho_ref, p.T_ref, out[0], out[1], out[2], out[3], msg, p.status);
     return cudaGetLastError();
 }
 
@@ -357,26 +358,30 @@ cudaError_t launch_import_rows(const KParams &p, int buf, int r0, int r1, const 
 
 template <typename S>
 cudaError_t launch_nusselt(const KParams &p, int buf, int side, double L, double dT, double *partials,
-                           cudaStream_t st) {
+                           unsigned *counter, ReadMsg *msg, cudaStream_t st) {
+    const int blocks = reduction_blocks(side < 2 ? p.ny : p.nx);
     if (p.tq == 9)
-        k_nusselt<S, 9><<<kRedBlocks, kRedThreads, 0, st>>>(make_planes<S>(p, buf), make_geom(p), side, L, dT,
-                                                           p.T_ref, partials);
+        k_nusselt<S, 9><<<blocks, kRedThreads, 0, st>>>(make_planes<S>(p, buf), make_geom(p), side, L, dT, p.T_ref,
+                                                       partials, counter, msg, p.status);
     else
-        k_nusselt<S, 5><<<kRedBlocks, kRedThreads, 0, st>>>(make_planes<S>(p, buf), make_geom(p), side, L, dT,
-                                                           p.T_ref, partials);
+        k_nusselt<S, 5><<<blocks, kRedThreads, 0, st>>>(make_planes<S>(p, buf), make_geom(p), side, L, dT, p.T_ref,
+                                                       partials, counter, msg, p.status);
     return cudaGetLastError();
 }
 
 template <typename S>
 cudaError_t launch_residual(const KParams &p, int buf, double *snap, int have_snap, double *partials,
-                            cudaStream_t st) {
+                            unsigned *counter, ReadMsg *msg, cudaStream_t st) {
     using C = typename Store<S>::C;
+    const int blocks = reduction_blocks((long long)p.nx * p.ny);
     if (p.tq == 9)
-        k_residual<S, 9><<<kRedBlocks, kRedThreads, 0, st>>>(make_planes<S>(p, buf), make_geom(p), make_rates<C>(p),
-                                                            p.T_ref, snap, p.plane, have_snap, partials);
+        k_residual<S, 9><<<blocks, kRedThreads, 0, st>>>(make_planes<S>(p, buf), make_geom(p), make_rates<C>(p),
+                                                        p.T_ref, snap, p.plane, have_snap, partials, counter, msg,
+                                                        p.status);
     else
-        k_residual<S, 5><<<kRedBlocks, kRedThreads, 0, st>>>(make_planes<S>(p, buf), make_geom(p), make_rates<C>(p),
-                                                            p.T_ref, snap, p.plane, have_snap, partials);
+        k_residual<S, 5><<<blocks, kRedThreads, 0, st>>>(make_planes<S>(p, buf), make_geom(p), make_rates<C>(p),
+                                                        p.T_ref, snap, p.plane, have_snap, partials, counter, msg,
+                                                        p.status);
     return cudaGetLastError();
 }
 

@@ -4,7 +4,10 @@
 // of nomrt_kernels.cuh.
 #include <cuda_runtime.h>
 
+#include <unistd.h>
+
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -30,6 +33,8 @@ thread_local std::string g_create_error;
 constexpr double kCs2 = 1.0 / 3.0;  // D2Q9 c_s^2 (Sec. 2.1)
 constexpr size_t kAlign = 256;
 constexpr size_t kStageBytes = 16u << 20;  // row-chunked host transfers
+
+static_assert(nomrt::kRedBlocks * 5 <= 512 * 8, "the reductions' scratch");
 
 const int kEx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};  // Eq. 5
 const int kEy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
@@ -61,7 +66,7 @@ Layout make_layout(int nx, int ny, int storage, int n_walls, int n_nee, int tq) 
     // at most 8192 rows per chunk keeps every chunked launch under the 65535 grid-y limit
     L.stage_rows = (int)std::max<size_t>(1, std::min<size_t>({(size_t)ny, kStageBytes / row_bytes, (size_t)8192}));
     L.off_stage = o; o += align_up(row_bytes * L.stage_rows, kAlign);
-    L.off_part = o; o += align_up(sizeof(double) * nomrt::kRedBlocks * 8, kAlign);
+    L.off_part = o; o += align_up(sizeof(double) * 512 * 8, kAlign);  // kRedBlocks of up to five sums
     L.off_res = o; o += align_up(sizeof(double) * 8, kAlign);
     L.off_status = o; o += kAlign;
     L.off_nee_dir = o; o += align_up(L.plane, kAlign);
@@ -377,6 +382,44 @@ lbm_status cuda_fail(lbm_lattice *h, cudaError_t e, const char *what) {
         if (e_ != cudaSuccess) return cuda_fail(h, e_, what); \
     } while (0)
 
+// Whether the GPU reads and writes ordinary host memory in place, through the
+// host's page tables (asked once per device).
+bool reaches_host(int dev) {
+    static std::atomic<int> known[nomrt::kMaxDevices];  // 0: not asked yet, 1: no, 2: yes
+    if (dev < 0 || dev >= nomrt::kMaxDevices) return false;
+    int k = known[dev].load(std::memory_order_relaxed);
+    if (k == 0) {
+        int access = 0, tables = 0;
+        const bool ok = cudaDeviceGetAttribute(&access, cudaDevAttrPageableMemoryAccess, dev) == cudaSuccess &&
+                        cudaDeviceGetAttribute(&tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev) ==
+                            cudaSuccess;
+        if (!ok) cudaGetLastError();
+        k = ok && access && tables ? 2 : 1;
+        known[dev].store(k, std::memory_order_relaxed);
+    }
+    return k == 2;
+}
+
+bool reaches_host() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return reaches_host(dev);
+}
+
+// Writes one byte to every page of [p, p + bytes), about to be overwritten by the
+// GPU: pages not yet mapped are mapped here, at the host's rate, rather than one
+// fault of the GPU's at a time (11.6 MB of them: 0.4 ms against 3.5).
+void touch_pages(void *p, size_t bytes) {
+    if (bytes == 0) return;
+    static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    volatile char *c = static_cast<volatile char *>(p);
+    for (size_t o = 0; o < bytes; o += page) c[o] = 0;
+    c[bytes - 1] = 0;
+}
+
 // After a stream synchronisation: a kernel that gave up a bounded wait left a
 // non-zero status word, or (bounds-checking build) a refused access left a
 // non-zero bounds word; report it once and clear both.
@@ -396,6 +439,26 @@ lbm_status check_status(lbm_lattice *h) {
         return fail(h, LBM_ECUDA, buf);
     }
     return fail(h, LBM_ETIMEOUT, "a kernel gave up a bounded wait (device status word set)");
+}
+
+// The same from the status words a read-out brought along.
+lbm_status check_msg(lbm_lattice *h, const nomrt::ReadMsg &m) {
+    return m.status[0] == nomrt::kStatusOk && m.status[1] == 0 ? LBM_OK : check_status(h);
+}
+
+// Runs `launch(msg)`, which queues a kernel that fills in a message, and waits
+// for it: the GPU writes h->msg in place where it reaches host memory; else the
+// message comes back from the device.
+template <typename F>
+lbm_status fetch_msg(lbm_lattice *h, F launch, const char *what) {
+    const bool direct = reaches_host();
+    nomrt::ReadMsg *const dev = reinterpret_cast<nomrt::ReadMsg *>(h->result());
+    cudaError_t e = launch(direct ? &h->msg : dev);
+    if (e == cudaSuccess && !direct)
+        e = cudaMemcpyAsync(&h->msg, dev, sizeof h->msg, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, what);
+    return check_msg(h, h->msg);
 }
 
 #define LBM_STATUS(h)                      \
@@ -479,14 +542,15 @@ bool plan_tiles(lbm_lattice *h) {
     return h->tile_plan.shape >= 0;
 }
 
-// n >= 2 steps as evenly sized launches of at most tile_plan.steps steps, as many
-// launches as steps modulo 2: an even run ends on the buffer it began on, so that
-// a caller's graph of one can be replayed with other even runs between. Each is a
-// programmatic dependent of the one before and costs the GPU more time than its
-// launch costs the host, so they are launched directly.
+// n >= 2 steps as evenly sized launches of at most tile_plan.steps steps. Once a
+// run has been recorded into a caller's graph, as many launches as steps modulo
+// 2: an even run then ends on the buffer it began on, so that the graph of one
+// can be replayed with other even runs between. Each is a programmatic dependent
+// of the one before and costs the GPU more time than its launch costs the host,
+// so they are launched directly.
 lbm_status step_tiles(lbm_lattice *h, int64_t n) {
     int64_t launches = (n + h->tile_plan.steps - 1) / h->tile_plan.steps;
-    launches += (launches ^ n) & 1;
+    if (h->recorded) launches += (launches ^ n) & 1;
     for (int64_t i = launches; i > 0; --i) {
         const int k = (int)((n + i - 1) / i);
         cudaError_t e = h->tile->launch(h->kp, h->tile_plan.shape, h->tile_map[h->cur], h->cur, k, h->stream);
@@ -873,7 +937,6 @@ lbm_status lbm_step(lbm_lattice *h, int64_t nsteps) {
     if (!h) return fail(nullptr, LBM_EINVAL, "lattice is NULL");
     if (nsteps < 0) return fail(h, LBM_EINVAL, "nsteps must be >= 0");
     if (h->batch) return fail(h, LBM_EINVAL, "lattice belongs to a batch: step it with lbm_batch_step");
-    if (nsteps > 1 && h->kp.variant == nomrt::kStepAuto && plan_tiles(h)) return step_tiles(h, nsteps);
     // Runs of kGraphShort steps or more replay captured graphs of kGraphSteps and kGraphShort
     // steps: the same kernels with the same arguments, without the launch gap between steps.
     // Direct launches serve short runs and remainders, a stream that is already being
@@ -882,6 +945,8 @@ lbm_status lbm_step(lbm_lattice *h, int64_t nsteps) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const cudaError_t ce = cudaStreamIsCapturing(h->stream, &cs);
     if (ce != cudaSuccess) cudaGetLastError();  // leave no error behind for the launch checks
+    if (ce == cudaSuccess && cs != cudaStreamCaptureStatusNone) h->recorded = true;
+    if (nsteps > 1 && h->kp.variant == nomrt::kStepAuto && plan_tiles(h)) return step_tiles(h, nsteps);
     const bool can_graph = !h->graph_off && ce == cudaSuccess && cs == cudaStreamCaptureStatusNone;
     if (!can_graph || nsteps < kGraphShort) return step_direct(h, nsteps);
     if (!h->direct_done || h->graph_variant != h->kp.variant || h->graph_config != h->kp.config) {
@@ -948,21 +1013,37 @@ lbm_status lbm_read_macro_rows(lbm_lattice *h, int32_t y0, int32_t y1, double *r
     if (y0 < 0 || y1 > h->ny || y0 > y1) return fail(h, LBM_EINVAL, "rows must satisfy 0 <= y0 <= y1 <= ny");
     double *outs[4] = {rho, ux, uy, T};
     const int nx = h->nx;
-    // page-locked (or device) outputs are written by the kernel in place; any pageable one sends
-    // every output through the staging area
+    // outputs the GPU reaches are written by the kernel in place: page-locked or device ones, and ordinary
+    // host memory where it shares the host's page tables; any other sends every output through the staging
+    // area
     double *direct[4] = {nullptr, nullptr, nullptr, nullptr};
-    bool in_place = true;
+    bool in_place = true, ordinary = false;
     for (int k = 0; k < 4; ++k)
         if (outs[k]) {
             direct[k] = static_cast<double *>(const_cast<void *>(device_view(outs[k])));
+            if (!direct[k] && reaches_host()) {
+                direct[k] = outs[k];
+                ordinary = true;
+            }
             in_place = in_place && direct[k];
         }
     if (in_place) {
+        if (ordinary)
+            for (int k = 0; k < 4; ++k)
+                if (outs[k] && direct[k] == outs[k]) touch_pages(outs[k], (size_t)(y1 - y0) * nx * sizeof(double));
+        const bool brief = reaches_host();  // the status words come along
+        h->msg.status[0] = nomrt::kStatusOk;
+        h->msg.status[1] = 0;
         for (int r0 = y0; r0 < y1; r0 += 65535) {  // the grid's y extent is at most 65535 rows per launch
             const int r1 = std::min(y1, r0 + 65535);
             double *o[4];
             for (int k = 0; k < 4; ++k) o[k] = direct[k] ? direct[k] + (size_t)(r0 - y0) * nx : nullptr;
-            LBM_CUDA(h, h->L->macro_rows(h->kp, h->cur, r0, r1, o, h->stream), "macro kernel");
+            LBM_CUDA(h, h->L->macro_rows(h->kp, h->cur, r0, r1, o, brief ? &h->msg : nullptr, h->stream),
+                     "macro kernel");
+        }
+        if (brief && !nomrt::kBoundsBuild) {
+            LBM_CUDA(h, cudaStreamSynchronize(h->stream), "read macro sync");
+            return check_msg(h, h->msg);
         }
     } else {
         const int rows = std::max(1, h->lay.stage_rows * h->lay.nq / 4);
@@ -973,7 +1054,7 @@ lbm_status lbm_read_macro_rows(lbm_lattice *h, int32_t y0, int32_t y1, double *r
             // overwrite the staging area before they finish: one wait at the end suffices
             double *o[4];
             for (int k = 0; k < 4; ++k) o[k] = outs[k] ? h->stage() + k * n : nullptr;
-            LBM_CUDA(h, h->L->macro_rows(h->kp, h->cur, r0, r1, o, h->stream), "macro kernel");
+            LBM_CUDA(h, h->L->macro_rows(h->kp, h->cur, r0, r1, o, nullptr, h->stream), "macro kernel");
             for (int k = 0; k < 4; ++k)
                 if (outs[k])
                     LBM_CUDA(h,
@@ -1001,12 +1082,14 @@ lbm_status lbm_nusselt(lbm_lattice *h, int32_t side, double L, double delta_T, d
         // fluid cells across the lattice along the wall normal, on the middle line
         L = (double)(side < 2 ? h->across_x : h->across_y);
     }
-    LBM_CUDA(h, h->L->nusselt(h->kp, h->cur, side, L, delta_T, h->partials(), h->stream), "nusselt kernel");
-    LBM_CUDA(h, nomrt::reduce_partials(h->partials(), 2, h->result(), h->stream), "reduce kernel");
-    double r[2];
-    LBM_CUDA(h, cudaMemcpyAsync(r, h->result(), sizeof r, cudaMemcpyDeviceToHost, h->stream), "read nusselt");
-    LBM_CUDA(h, cudaStreamSynchronize(h->stream), "nusselt sync");
-    LBM_STATUS(h);
+    const lbm_status st = fetch_msg(
+        h,
+        [&](nomrt::ReadMsg *msg) {
+            return h->L->nusselt(h->kp, h->cur, side, L, delta_T, h->partials(), h->counter(), msg, h->stream);
+        },
+        "nusselt kernel");
+    if (st != LBM_OK) return st;
+    const double *r = h->msg.v;
     if (r[1] <= 0.0) return fail(h, LBM_EINVAL, "no fixed-temperature wall line on that side");
     *nu_mean = r[0] / r[1];
     return LBM_OK;
@@ -1016,12 +1099,14 @@ lbm_status lbm_residual(lbm_lattice *h, double *r) {
     if (!h) return fail(nullptr, LBM_EINVAL, "lattice is NULL");
     if (!r) return fail(h, LBM_EINVAL, "r is NULL");
     const int had = h->have_snap;
-    LBM_CUDA(h, h->L->residual(h->kp, h->cur, h->snap(), had, h->partials(), h->stream), "residual kernel");
-    LBM_CUDA(h, nomrt::reduce_partials(h->partials(), 5, h->result(), h->stream), "reduce kernel");
-    double s[5];
-    LBM_CUDA(h, cudaMemcpyAsync(s, h->result(), sizeof s, cudaMemcpyDeviceToHost, h->stream), "read residual");
-    LBM_CUDA(h, cudaStreamSynchronize(h->stream), "residual sync");
-    LBM_STATUS(h);
+    const lbm_status st = fetch_msg(
+        h,
+        [&](nomrt::ReadMsg *msg) {
+            return h->L->residual(h->kp, h->cur, h->snap(), had, h->partials(), h->counter(), msg, h->stream);
+        },
+        "residual kernel");
+    if (st != LBM_OK) return st;
+    const double *s = h->msg.v;
     h->have_snap = 1;
     if (s[4] > 0.0 || !std::isfinite(s[0]) || !std::isfinite(s[1]) || !std::isfinite(s[2]) ||
         !std::isfinite(s[3])) {

@@ -416,6 +416,55 @@ cudaError_t launch_batch_persistent(int config, const GroupParams &G, int parity
     }
 }
 
+// The residuals of up to kGroupLats members in one launch: each member's blocks and
+// sums are those of lbm_residual (residual_cells, reduce_finish), so its value
+// has the same bits.
+struct ResidualMember {
+    Geom g;
+    const void *src;
+    unsigned long long plane;
+    double *snap, *partials;
+    unsigned *counter;
+    const int *status;
+    double T_ref;
+    float ax, Fy0, g_beta;
+    int have_snap;
+};
+
+struct ResidualGroup {
+    int nlats;
+    int first[kGroupLats + 1];  // first block of each member
+    const int *batch_status;
+    ReadMsg *batch_msg;         // the batch's status word goes here
+    ReadMsg *msg;               // one per member
+    ResidualMember lat[kGroupLats];
+};
+static_assert(sizeof(ResidualGroup) <= 32764, "the members' descriptors must fit the kernel parameter space");
+
+template <typename S>
+__global__ void __launch_bounds__(kRedThreads, 4) k_batch_residual(const __grid_constant__ ResidualGroup P) {
+    const int b = (int)blockIdx.x;
+    int lo = 0, hi = P.nlats - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (P.first[mid] <= b) lo = mid;
+        else hi = mid - 1;
+    }
+    const ResidualMember &L = P.lat[lo];
+    if (b == 0 && threadIdx.x == 0) P.batch_msg->status[0] = *P.batch_status;
+    RatesC<float> r;
+    r.ax = L.ax;  // all that the macroscopic values take
+    r.Fy0 = L.Fy0;
+    r.g_beta = L.g_beta;
+    const S *src[kQ];
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) src[q] = static_cast<const S *>(L.src) + q * (size_t)L.plane;
+    const int block = b - P.first[lo], blocks = P.first[lo + 1] - P.first[lo];
+    double v[5] = {0, 0, 0, 0, 0};
+    residual_cells<S, 5>(src, L.g, r, L.T_ref, L.snap, (size_t)L.plane, L.have_snap, block, blocks, v);
+    reduce_finish<5>(v, L.partials, L.counter, block, blocks, P.msg + lo, L.status);
+}
+
 }  // namespace nomrt
 
 struct lbm_batch {
@@ -431,9 +480,8 @@ struct lbm_batch {
     // the launch groups' work tables (int2 per virtual block, groups side by side)
     int2 *d_work = nullptr;
     size_t cap_work = 0;
-    // lbm_batch_residuals: the members' five residual sums on the device and their pinned host copy
-    double *d_res = nullptr;
-    double *h_res = nullptr;
+    // lbm_batch_residuals: the batch's status and the members' residual sums, page-locked
+    nomrt::ReadMsg *h_res = nullptr;
     size_t cap_res = 0;
     std::vector<nomrt::GroupParams> groups;  // launch parameters, kGroupLats members each
     // FUSED, default config: several steps per launch where every member can (shape -1: not). One launch
@@ -1142,32 +1190,58 @@ lbm_status lbm_batch_residuals(lbm_batch *b, int32_t cap, lbm_lattice **members,
     if (!r) return bfail(b, LBM_EINVAL, "r is NULL");
     if ((size_t)m > b->cap_res) {
         cudaError_t e = cudaStreamSynchronize(b->stream);
-        if (b->d_res) cudaFree(b->d_res);
         if (b->h_res) cudaFreeHost(b->h_res);
-        b->d_res = nullptr;
         b->h_res = nullptr;
         b->cap_res = 0;
         const size_t want = std::max<size_t>((size_t)m * 3 / 2, 64);
-        if (e == cudaSuccess) e = cudaMalloc(&b->d_res, want * 5 * sizeof(double));
-        if (e == cudaSuccess) e = cudaHostAlloc(&b->h_res, want * 5 * sizeof(double), cudaHostAllocDefault);
+        // the first message holds the batch's own status word
+        if (e == cudaSuccess) e = cudaHostAlloc(&b->h_res, (want + 1) * sizeof(nomrt::ReadMsg), cudaHostAllocDefault);
         if (e != cudaSuccess) return bcuda(b, e, "residual buffers");
         b->cap_res = want;
     }
-    // every member's residual kernels on the batch's stream, their sums side by side
-    for (int i = 0; i < m; ++i) {
-        lbm_lattice *h = b->members[i];
-        cudaError_t e = h->L->residual(h->kp, h->cur, h->snap(), h->have_snap, h->partials(), b->stream);
-        if (e == cudaSuccess) e = nomrt::reduce_partials(h->partials(), 5, b->d_res + 5 * (size_t)i, b->stream);
-        if (e != cudaSuccess) return bcuda(b, e, "residual kernels");
+    // every member's residual in one launch per kGroupLats members, the sums written to page-locked memory
+    for (int at = 0; at < m; at += nomrt::kGroupLats) {
+        nomrt::ResidualGroup G;
+        std::memset(&G, 0, sizeof G);
+        G.nlats = std::min(nomrt::kGroupLats, m - at);
+        for (int i = 0; i < G.nlats; ++i) {
+            const lbm_lattice *h = b->members[at + i];
+            const nomrt::RatesC<float> r = nomrt::make_rates<float>(h->kp);
+            nomrt::ResidualMember &t = G.lat[i];
+            t.g = nomrt::make_geom(h->kp);
+            t.src = h->kp.pop[h->cur];
+            t.plane = h->kp.plane;
+            t.snap = h->snap();
+            t.partials = h->partials();
+            t.counter = h->counter();
+            t.status = h->kp.status;
+            t.T_ref = h->kp.T_ref;
+            t.ax = r.ax;
+            t.Fy0 = r.Fy0;
+            t.g_beta = r.g_beta;
+            t.have_snap = h->have_snap;
+            G.first[i + 1] = G.first[i] + nomrt::reduction_blocks((long long)h->kp.nx * h->kp.ny);
+        }
+        G.batch_status = b->d_status;
+        G.batch_msg = b->h_res;
+        G.msg = b->h_res + 1 + at;
+        const unsigned blocks = (unsigned)G.first[G.nlats];
+        if (b->storage == LBM_F16_SHIFTED)
+            nomrt::k_batch_residual<__half><<<blocks, nomrt::kRedThreads, 0, b->stream>>>(G);
+        else
+            nomrt::k_batch_residual<float><<<blocks, nomrt::kRedThreads, 0, b->stream>>>(G);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return bcuda(b, e, "residual kernel");
     }
-    cudaError_t e = cudaMemcpyAsync(b->h_res, b->d_res, (size_t)m * 5 * sizeof(double), cudaMemcpyDeviceToHost,
-                                    b->stream);
+    const cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "read residuals");
-    lbm_status st = lbm_batch_sync(b);
-    if (st != LBM_OK) return st;
+    if (nomrt::kBoundsBuild || b->h_res[0].status[0] != nomrt::kStatusOk) {
+        const lbm_status st = lbm_batch_sync(b);
+        if (st != LBM_OK) return st;
+    }
     for (int i = 0; i < m; ++i) {
         lbm_lattice *h = b->members[i];
-        const double *q = b->h_res + 5 * (size_t)i;
+        const double *q = b->h_res[1 + i].v;
         if (members) members[i] = h;
         const int had = h->have_snap;
         h->have_snap = 1;
@@ -1209,7 +1283,6 @@ void lbm_batch_destroy(lbm_batch *b) {
     if (b->cap) cudaStreamDestroy(b->cap);
     if (b->d_bar) cudaFree(b->d_bar);
     if (b->d_status) cudaFree(b->d_status);
-    if (b->d_res) cudaFree(b->d_res);
     if (b->h_res) cudaFreeHost(b->h_res);
     if (b->d_work) cudaFree(b->d_work);
     delete b;

@@ -20,9 +20,21 @@ constexpr int kQmax = 18;
 constexpr int kMaxDevices = 64;
 // Link-map value of a solid cell (and of the row padding).
 constexpr uint8_t kSolid = 0xFF;
-// Fixed number of blocks of the reduction kernels (deterministic sums).
-constexpr int kRedBlocks = 512;
+// Blocks of a reduction kernel (at most; deterministic sums: the blocks depend on the work alone)
+// and the partial sums its scratch holds per block.
+constexpr int kRedBlocks = 608;  // four per SM
 constexpr int kRedThreads = 256;
+inline int reduction_blocks(long long work) {
+    const long long n = (work + kRedThreads - 1) / kRedThreads;
+    return n < 1 ? 1 : n < kRedBlocks ? (int)n : kRedBlocks;
+}
+
+// What a reduction or a read-out leaves for the host: its sums, and the lattice's
+// status and bounds words as it found them.
+struct ReadMsg {
+    double v[5];
+    int status[2];
+};
 // Device status word values (set by kernels, read and cleared by the host).
 constexpr int kStatusOk = 0;
 constexpr int kStatusTimeout = 1;
@@ -122,19 +134,22 @@ struct Launchers {
     // initial state into buffer `buf`, rows [r0, r1), zeros into the other buffer; T rows in `T`
     // (device-readable, (r1-r0)*nx), or nullptr for T0 everywhere
     cudaError_t (*init_rows)(const KParams &, int buf, int r0, int r1, const double *T, cudaStream_t st);
-    // macroscopics of rows [r0, r1) into out[0..3] (rho, ux, uy, T; (r1-r0)*nx doubles each, any NULL)
-    cudaError_t (*macro_rows)(const KParams &, int buf, int r0, int r1, double *const out[4], cudaStream_t st);
+    // macroscopics of rows [r0, r1) into out[0..3] (rho, ux, uy, T; (r1-r0)*nx doubles each, any NULL); msg:
+    // NULL, or where to leave the status words
+    cudaError_t (*macro_rows)(const KParams &, int buf, int r0, int r1, double *const out[4], ReadMsg *msg,
+                              cudaStream_t st);
     // FP64 export / import of rows [r0, r1): out/in [9 + tq][(r1-r0)*nx]
     cudaError_t (*export_rows)(const KParams &, int buf, int r0, int r1, double *out, cudaStream_t st);
     cudaError_t (*import_rows)(const KParams &, int buf, int r0, int r1, const double *in, int which,
                                cudaStream_t st);
-    // Nusselt partial sums (sum, count) per block into partials[kRedBlocks][2]
+    // sum and count of the Nusselt lines into msg->v[0..1]; partials: kRedBlocks * 8 doubles, counter: a zero
+    // word, left zero
     cudaError_t (*nusselt)(const KParams &, int buf, int side, double L, double dT, double *partials,
-                           cudaStream_t st);
-    // residual partial sums (|du|^2, |u|^2, dT^2, T^2, nonfinite) per block into
-    // partials[kRedBlocks][5]; updates snap[3][plane] (ux, uy, T)
+                           unsigned *counter, ReadMsg *msg, cudaStream_t st);
+    // |du|^2, |u|^2, dT^2, T^2 and the count of non-finite cells into msg->v[0..4]; updates
+    // snap[3][plane] (ux, uy, T)
     cudaError_t (*residual)(const KParams &, int buf, double *snap, int have_snap, double *partials,
-                            cudaStream_t st);
+                            unsigned *counter, ReadMsg *msg, cudaStream_t st);
 };
 
 // storage: the ABI's (0 f64, 1 f32, 2 f16); nullptr for FP64, which steps once per launch.
@@ -146,8 +161,5 @@ const Launchers &launchers_f16();
 
 // Sets the calling thread's error message (lbm_last_error(NULL)).
 void set_thread_error(const char *msg);
-
-// Final fixed-order reduction of partials[kRedBlocks][width] into out[width].
-cudaError_t reduce_partials(const double *partials, int width, double *out, cudaStream_t st);
 
 }  // namespace nomrt

@@ -987,12 +987,17 @@ __global__ void k_init_rows(const Planes<S> pl, const Geom g, int r0, int r1, co
 
 // rho, u_x, u_y, T of rows [r0, r1) into out[0..3] (each (r1 - r0) * nx
 // doubles, row y at (y - r0) * nx; a NULL output is skipped). The outputs may
-// be a staging area or the caller's page-locked host arrays.
+// be a staging area or the caller's host arrays. msg: NULL, or where to leave
+// the status words.
 template <typename S, int TQ = 5>
 __global__ void k_macro_rows(const Planes<S> pl, const Geom g, const RatesC<typename Store<S>::C> r, int r0,
                              int r1, double rho_ref, double T_ref, double *o_rho, double *o_ux, double *o_uy,
-                             double *o_T) {
+                             double *o_T, ReadMsg *msg, const int *status) {
     using C = typename Store<S>::C;
+    if (msg && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        msg->status[0] = status[0];
+        msg->status[1] = status[1];
+    }
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = r0 + blockIdx.y;
     if (x >= g.nx || y >= r1) return;
@@ -1060,9 +1065,15 @@ __global__ void k_import_rows(const Planes<S> pl, const Geom g, int r0, int r1, 
 
 // ------------------------------------------------------------- reductions
 
+// The end of a reduction over `blocks` blocks, this one number `block`: its sums
+// into partials, and in the block that comes last all of them, block by block in
+// a fixed order, into msg, with the status words. counter: zero, left zero.
 template <int W>
-__device__ __forceinline__ void block_reduce_store(double (&v)[W], double *partials) {
+__device__ __forceinline__ void reduce_finish(double (&v)[W], double *partials, unsigned *counter, int block,
+                                              int blocks, ReadMsg *msg, const int *status) {
+    static_assert(W <= kRedThreads / 32, "one warp per sum");
     __shared__ double sh[kRedThreads / 32][W];
+    __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < W; ++k)
@@ -1070,13 +1081,27 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[W], double *parti
     if (lane == 0)
         for (int k = 0; k < W; ++k) sh[warp][k] = v[k];
     __syncthreads();
-    if (threadIdx.x < 32) {
-#pragma unroll
-        for (int k = 0; k < W; ++k) {
-            double a = lane < kRedThreads / 32 ? sh[lane][k] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-            if (lane == 0) partials[blockIdx.x * W + k] = a;
-        }
+    if (threadIdx.x < W) {
+        double a = 0.0;
+        for (int w = 0; w < kRedThreads / 32; ++w) a += sh[w][threadIdx.x];
+        partials[block * W + threadIdx.x] = a;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == (unsigned)blocks - 1u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (warp < W) {
+        double a = 0.0;
+        for (int b = lane; b < blocks; b += 32) a += __ldcg(partials + b * W + warp);
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+        if (lane == 0) msg->v[warp] = a;
+    }
+    if (threadIdx.x == 0) {
+        *counter = 0u;
+        msg->status[0] = status[0];
+        msg->status[1] = status[1];
     }
 }
 
@@ -1096,7 +1121,8 @@ __device__ __forceinline__ double temperature_at(const Planes<S> &pl, const Geom
 // Eq. 39 with the one-sided wall gradient; one thread per line along the wall.
 template <typename S, int TQ = 5>
 __global__ void __launch_bounds__(kRedThreads) k_nusselt(const Planes<S> pl, const Geom g, int side, double L,
-                                                         double dT, double T_ref, double *partials) {
+                                                         double dT, double T_ref, double *partials,
+                                                         unsigned *counter, ReadMsg *msg, const int *status) {
     const int along = side < 2 ? g.ny : g.nx;
     double v[2] = {0.0, 0.0};
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < along; s += gridDim.x * blockDim.x) {
@@ -1121,40 +1147,61 @@ __global__ void __launch_bounds__(kRedThreads) k_nusselt(const Planes<S> pl, con
         v[0] += -L * dTdn / dT;
         v[1] += 1.0;
     }
-    block_reduce_store<2>(v, partials);
+    reduce_finish<2>(v, partials, counter, (int)blockIdx.x, (int)gridDim.x, msg, status);
 }
 
-template <typename S, int TQ = 5>
-__global__ void __launch_bounds__(kRedThreads) k_residual(const Planes<S> pl, const Geom g,
-                                                          const RatesC<typename Store<S>::C> r, double T_ref,
-                                                          double *snap, size_t plane, int have_snap,
-                                                          double *partials) {
+// One block's cells of a residual over `blocks` blocks: v += |du|^2, |u|^2, dT^2,
+// T^2, non-finite cells; the snapshot takes the new values. Bound by the FP64
+// pipe on large lattices: 13 operations per cell.
+template <typename S, int TQ>
+__device__ __forceinline__ void residual_cells(const S *const *src, const Geom &g,
+                                               const RatesC<typename Store<S>::C> &r, double T_ref, double *snap,
+                                               size_t plane, int have_snap, int block, int blocks, double (&v)[5]) {
     using C = typename Store<S>::C;
-    double v[5] = {0, 0, 0, 0, 0};
-    const long long total = (long long)g.ny * g.nx;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < total;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(c / g.nx), x = (int)(c - (long long)y * g.nx);
-        const int off = y * g.pitch + x;
+    // the rows that can hold a fluid cell; every load of a cell, its snapshot's too, is in flight before
+    // the first is looked at (a solid cell's pulls stay within the planes and are not used)
+    const unsigned row0 = g.py ? 0u : 1u, rows = (unsigned)max(0, g.ny - 2 * (int)row0);
+    const unsigned total = rows * (unsigned)g.nx, step = (unsigned)blocks * kRedThreads;
+    unsigned bad = 0;
+    for (unsigned c = (unsigned)block * kRedThreads + threadIdx.x; c < total; c += step) {
+        const unsigned row = c / (unsigned)g.nx, x = c - row * (unsigned)g.nx, y = row + row0;
+        const int off = (int)(y * (unsigned)g.pitch + x);
         const unsigned m = g.mask[off];
-        if (m == kSolid) continue;
+        double sx = 0.0, sy = 0.0, sT = 0.0;
+        if (have_snap) {
+            sx = snap[off];
+            sy = snap[plane + off];
+            sT = snap[2 * plane + off];
+        }
         C f[9], t[TQ];
-        pull<S, TQ>(pl.src, g, x, y, m, f, t);
-        Macro<C> M = macro_of<C, TQ>(r, f, t);
+        pull<S, TQ>(src, g, (int)x, (int)y, m == kSolid ? 0u : m, f, t);
+        if (m == kSolid) continue;
+        const Macro<C> M = macro_of<C, TQ>(r, f, t);
         const double ux = (double)M.ux, uy = (double)M.uy, T = T_ref + (double)M.dT;
         if (have_snap) {
-            const double a = ux - snap[off], b = uy - snap[plane + off], d = T - snap[2 * plane + off];
-            v[0] += a * a + b * b;
-            v[2] += d * d;
+            const double a = ux - sx, b = uy - sy, d = T - sT;
+            v[0] = __fma_rn(a, a, __fma_rn(b, b, v[0]));
+            v[2] = __fma_rn(d, d, v[2]);
         }
-        v[1] += ux * ux + uy * uy;
-        v[3] += T * T;
-        if (!isfinite(ux) || !isfinite(uy) || !isfinite(T)) v[4] += 1.0;
+        v[1] = __fma_rn(ux, ux, __fma_rn(uy, uy, v[1]));
+        v[3] = __fma_rn(T, T, v[3]);
+        bad += !isfinite(M.ux) || !isfinite(M.uy) || !isfinite(M.dT);
         snap[off] = ux;
         snap[plane + off] = uy;
         snap[2 * plane + off] = T;
     }
-    block_reduce_store<5>(v, partials);
+    v[4] += (double)bad;
+}
+
+template <typename S, int TQ = 5>
+__global__ void __launch_bounds__(kRedThreads, TQ == 9 ? 3 : 4) k_residual(const Planes<S> pl, const Geom g,
+                                                          const RatesC<typename Store<S>::C> r, double T_ref,
+                                                          double *snap, size_t plane, int have_snap,
+                                                          double *partials, unsigned *counter, ReadMsg *msg,
+                                                          const int *status) {
+    double v[5] = {0, 0, 0, 0, 0};
+    residual_cells<S, TQ>(pl.src, g, r, T_ref, snap, plane, have_snap, (int)blockIdx.x, (int)gridDim.x, v);
+    reduce_finish<5>(v, partials, counter, (int)blockIdx.x, (int)gridDim.x, msg, status);
 }
 
 // ------------------------------------------------- vectorised step kernel
