@@ -38,10 +38,13 @@ inline TileCover tile_cover(const KParams &p) {
 // to 8 steps on lattices of 64^2 to 4096 x 2048 cells and on batches of 24 to
 // 64 cavities (rms error 13 %); the shape and steps it picks run within 2 % of
 // the fastest of them but for 180^2 cells (19 %).
-inline double tile_cycles(const TileShape &s, int k, long long tiles, double cell_bytes, bool fits_l2, int sms) {
-    constexpr double kLaunch = 11600, kLatency = 920, kRound = 1.18;
+inline double tile_cycles(const TileShape &s, int k, long long tiles, int nq, double cell_bytes, bool fits_l2,
+                          int sms) {
+    constexpr double kLaunch = 11600, kRound = 1.18;
     constexpr double kTogether[4] = {153, 141, 142, 125};  // cycles per 32 pairs with 1..4 blocks on the SM
-    constexpr double kBlock = 3640, kPairWarp = 80.3, kWarpStep = 8.1, kHbm = 21.2;  // many waves; bytes per cycle and SM
+    constexpr double kBlock = 3640, kWarpStep = 8.1, kHbm = 21.2;  // many waves; bytes per cycle and SM
+    // a pair's cost goes with its populations (fitted with 14)
+    const double scale = nq / 14.0, kLatency = 920 * scale, kPairWarp = 80.3 * scale;
     double pair_warps = 0;
     const int cols = shape_cols(s, k), rows = shape_rows(s, k);
     auto pairs = [&](int l) { return (s.ry / 2 - l) * (l < k ? s.rx : cols); };
@@ -51,7 +54,7 @@ inline double tile_cycles(const TileShape &s, int k, long long tiles, double cel
         for (int l = 1; l <= k; ++l) {
             const int rounds = (pairs(l) + s.threads - 1) / s.threads;
             t += std::max(kLatency * (1 + kRound * (rounds - 1)),
-                          n * ((pairs(l) + 31) / 32) * kTogether[std::min(n, 4) - 1]);
+                          n * ((pairs(l) + 31) / 32) * scale * kTogether[std::min(n, 4) - 1]);
         }
         return t;
     };
@@ -102,7 +105,7 @@ inline TilePlan choose_tile(const KParams *const *lats, int n, int nq, int elem,
                 tiles += gx * gy;
             }
             if (!fits || tiles > 0x3FFFFFFF) continue;
-            const double t = tile_cycles(shapes[i], k, tiles, cell_bytes, fits_l2, sms) / k;
+            const double t = tile_cycles(shapes[i], k, tiles, nq, cell_bytes, fits_l2, sms) / k;
             if (best.shape < 0 || t < least) {
                 best = TilePlan{i, k};
                 least = t;
