@@ -442,7 +442,7 @@ struct ResidualGroup {
 static_assert(sizeof(ResidualGroup) <= 32764, "the members' descriptors must fit the kernel parameter space");
 
 template <typename S>
-__global__ void __launch_bounds__(kRedThreads, 4) k_batch_residual(const __grid_constant__ ResidualGroup P) {
+__global__ void __launch_bounds__(kRedThreads) k_batch_residual(const __grid_constant__ ResidualGroup P) {
     const int b = (int)blockIdx.x;
     int lo = 0, hi = P.nlats - 1;
     while (lo < hi) {

@@ -90,10 +90,10 @@ __device__ constexpr int kTileEx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
 __device__ constexpr int kTileEy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
 __device__ constexpr int kTileOpp[9] = {0, 3, 4, 1, 2, 7, 8, 5, 6};
 
-// The value a population has after one trip through the storage.
+// The values two cells' populations have after one trip through the storage.
 template <typename S>
-__device__ __forceinline__ float stored(float v) {
-    if constexpr (sizeof(S) == 2) return __half2float(__float2half_rn(v));
+__device__ __forceinline__ float2 stored(float2 v) {
+    if constexpr (sizeof(S) == 2) return __half22float2(__float22half2_rn(v));
     else return v;
 }
 
@@ -185,14 +185,6 @@ __device__ __forceinline__ void tile_copy_half(float *to, const CUtensorMap *map
         "[%2];" ::"r"(smem_u32(to)),
         "l"(map), "r"(smem_u32(bar)), "r"(gx), "r"((gy - par) / 2), "r"(par), "r"(0)
         : "memory");
-}
-
-// Asks L2 for one half of a region a later block will copy.
-__device__ __forceinline__ void tile_prefetch_half(const CUtensorMap *map, int gx, int gy) {
-    const int par = gy & 1;
-    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(map), "r"(gx),
-                 "r"((gy - par) / 2), "r"(par), "r"(0)
-                 : "memory");
 }
 
 // FP16: the region's cells on the lattice, four at a time, as their FP32 images
@@ -342,9 +334,9 @@ __device__ __forceinline__ void tile_pass(const PA &pl, const Geom &g, const Rat
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) f[i] = make_float2(stored<S>(f[i].x), stored<S>(f[i].y));
+            for (int i = 0; i < 9; ++i) f[i] = stored<S>(f[i]);
 #pragma unroll
-            for (int i = 0; i < TQ; ++i) t[i] = make_float2(stored<S>(t[i].x), stored<S>(t[i].y));
+            for (int i = 0; i < TQ; ++i) t[i] = stored<S>(t[i]);
 #pragma unroll
             for (int i = 0; i < 9 + TQ; ++i) {
                 const int d = i < 9 ? i : i - 9;
@@ -428,19 +420,13 @@ __host__ __device__ constexpr int tile_cols(int k) { return (RX - tile_margin(k)
 template <int RY>
 __host__ __device__ constexpr int tile_rows(int k) { return RY - 2 * k; }
 
-// The first cell of a region to prefetch; gx0 <= -RX: none.
-struct TileAhead {
-    int gx0, gy0;
-};
-
 // k steps of the tile whose first output cell is (ox, oy), ox a multiple of 4.
 // map: the source buffer's tensor map (FP32). early: read what does not change
 // between steps before waiting for the previous launch (a grid whose blocks can
 // become resident before it ends).
 template <typename S, int TQ, bool BGK, int RX, int RY, int T, typename PA>
 __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const RatesC<float> &r, TileWalls walls,
-                                           const CUtensorMap *map, int k, int ox, int oy, bool early, TileAhead ahead,
-                                           int *status) {
+                                           const CUtensorMap *map, int k, int ox, int oy, bool early, int *status) {
     using Lay = TileLayout<TQ, RX, RY>;
     extern __shared__ __align__(128) float tile_smem[];
     uint64_t *const bar = reinterpret_cast<uint64_t *>(tile_smem);
@@ -495,19 +481,7 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     }
     if (!early) any = tile_maps<TQ, RX, RY, T>(g, maps, gx0, gy0);
     const bool walled = __syncthreads_or(any);  // also: the barrier is initialised
-    if (boxed) {
-        if (!mbar_wait_bounded(bar, 0)) *gave_up = 1;
-        // the region of the block that will follow this one on the SM: into L2 while this one computes
-        if (ahead.gx0 > -RX) {
-            if (threadIdx.x == 0) {
-                tile_prefetch_half(map, ahead.gx0, ahead.gy0);
-                tile_prefetch_half(map, ahead.gx0, ahead.gy0 + 1);
-            }
-            const int x = max(ahead.gx0, 0), y = ahead.gy0 + (int)threadIdx.x;
-            if (threadIdx.x < RY && y >= 0 && y < g.ny && NOMRT_OK(g, g.mask + (size_t)y * g.pitch + x, 1, 65))
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(g.mask + (size_t)y * g.pitch + x));
-        }
-    }
+    if (boxed && !mbar_wait_bounded(bar, 0)) *gave_up = 1;
     // a periodic x: the columns beyond the seam
     const int c1 = (g.nx & ~3) - gx0;
     if (rows && g.px && (gx0 < 0 || c1 < RX)) {
@@ -537,16 +511,10 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
 template <typename S, int TQ, bool BGK, int RX, int RY, int T, int MINB>
 __global__ void __launch_bounds__(T, MINB)
     k_tile(const Planes<S> pl, const Geom g, const RatesC<float> r, const __grid_constant__ CUtensorMap map,
-           TileWalls walls, int k, int row0, int early, int resident, int *status) {
+           TileWalls walls, int k, int row0, int early, int *status) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int b = (int)(blockIdx.y * gridDim.x + blockIdx.x) + resident;
-    TileAhead ahead{-RX, 0};
-    if (b < (int)(gridDim.x * gridDim.y)) {
-        const int by = b / (int)gridDim.x, bx = b - by * (int)gridDim.x;
-        ahead = TileAhead{bx * tile_cols<RX>(k) - tile_margin(k), row0 + by * tile_rows<RY>(k) - k};
-    }
     tile_steps<S, TQ, BGK, RX, RY, T>(pl, g, r, walls, &map, k, (int)blockIdx.x * tile_cols<RX>(k),
-                                      row0 + (int)blockIdx.y * tile_rows<RY>(k), early != 0, ahead, status);
+                                      row0 + (int)blockIdx.y * tile_rows<RY>(k), early != 0, status);
 }
 
 }  // namespace nomrt

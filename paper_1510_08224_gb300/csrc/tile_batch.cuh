@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(T, MINB) k_tile_batch(const __grid_constant__ 
     RatesC<float> r = P.rc;  // shared rates: parameter-bank operands
     apply_member(r, L.v);
     tile_steps<S, 5, false, RX, RY, T>(pl, g, r, L.walls, &L.map, P.k, bx * tile_cols<RX>(P.k),
-                                       L.row0 + by * tile_rows<RY>(P.k), P.early != 0, TileAhead{-RX, 0}, P.status);
+                                       L.row0 + by * tile_rows<RY>(P.k), P.early != 0, P.status);
 }
 
 // The several-steps-per-launch kernels of a batch (MRT, D2Q5).

@@ -167,8 +167,8 @@ inline size_t tile_smem_bytes(const TileShape &s, long long tiles, int sms) {
 }
 
 template <typename S>
-using TileKernel = void (*)(const Planes<S>, const Geom, const RatesC<float>, const CUtensorMap, TileWalls, int, int,
-                            int, int, int *);
+using TileKernel = void (*)(const Planes<S>, const Geom, const RatesC<float>, const CUtensorMap, TileWalls, int, int, int,
+                            int *);
 
 // The current device, the kernel's shared-memory limit raised on it once.
 template <typename K>
@@ -208,9 +208,9 @@ cudaError_t launch_tile(TileKernel<S> kern, const TileShape &s, std::atomic<bool
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const int resident = sms * s.per_sm;
     return cudaLaunchKernelEx(&cfg, kern, make_planes<S>(p, src), make_geom(p), make_rates<float>(p), map,
-                              TileWalls{p.n_walls, p.moving}, k, c.row0, (int)(tiles <= resident), resident, p.status);
+                              TileWalls{p.n_walls, p.moving}, k, c.row0, (int)(tiles <= (long long)sms * s.per_sm),
+                              p.status);
 }
 
 // The shapes of one storage, temperature lattice and collision: region columns
