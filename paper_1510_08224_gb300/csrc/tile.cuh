@@ -33,10 +33,13 @@
 // FP16 storage keeps its values in shared memory as the FP32 images of the
 // rounded ones, so a step gives the bits it gives through global memory.
 //
-// FP32 regions arrive through a tensor map, one bulk copy per row parity:
-// per-thread 16-byte copies and one bulk copy per row kept the load/store unit
-// or the copy engine busy for as long as the steps took (82 and 74 us a step at
-// 4096 x 2048 cells, the tensor map 66). The blocks of an SM are small enough
+// Regions arrive through a tensor map, one bulk copy per row parity: per-thread
+// 16-byte copies and one bulk copy per row kept the load/store unit or the copy
+// engine busy for as long as the steps took (82 and 74 us a step at 4096 x 2048
+// cells, the tensor map 66). FP16 halves land where the FP32 planes will be and
+// are expanded in place through registers (per-thread loads and conversions
+// instead: 27.2 us a step at 2048 x 1024, expanded copies 21.6, 20.2 with
+// regions of 40 x 32). The blocks of an SM are small enough
 // that three or four are resident: one copies while others compute. Tried
 // without gain: pulling the first step from global memory directly (86 us), 2
 // blocks of 72 x 26 cells (64), 288 to 448 threads (66: each thread sets up a
@@ -49,7 +52,8 @@
 // cycles) and of a launch. Measured, us per step, one step per launch -> this:
 // FP32 4096 x 2048 138 -> 60, 1024^2 22 -> 11, 600^2 7.0 -> 5.8, 128^2 5.5 ->
 // 1.4, 64^2 5.9 -> 1.2; with the D2Q9 temperature model 177 -> 88 at 4096 x
-// 2048; FP16 600^2 9.1 -> 5.7, 128^2 5.8 -> 1.5.
+// 2048; FP16 2048 x 1024 24.5 -> 20.2, 1024^2 14.1 -> 12.0, 600^2 9.1 -> 5.7,
+// 128^2 5.8 -> 1.5.
 #pragma once
 
 #include <cuda.h>
@@ -74,6 +78,11 @@ struct TileLayout {
     // first row's)
     static constexpr int HS = (NQ * PS + 31) / 32 * 32;
     static constexpr int kHead = 32;        // words before the planes: the copies' barrier
+    // FP16: the box a half arrives in (bytes), wide enough to start on a multiple of 8 cells
+    static constexpr int kHalfCols = RX + 8;
+    static constexpr int kHalfBox = NQ * (RY / 2) * kHalfCols * 2;
+    static constexpr int kHalfStride = (kHalfBox + 127) / 128 * 128;
+    static_assert(2 * kHalfStride <= 8 * HS, "the copied halves lie where the planes will");
     // the maps (bytes): one half after the other, with guard bytes around each
     static constexpr int kGuard = 4;
     static constexpr int MS = PS + kGuard;
@@ -178,7 +187,7 @@ __device__ __forceinline__ bool tile_maps(const Geom &g, uint8_t *maps, int gx0,
 // One half of the region (every second row, from lattice row gy) through the
 // source buffer's tensor map: x, row pair, row parity, plane. Rows and columns
 // off the lattice arrive as zeros or as the padding's values.
-__device__ __forceinline__ void tile_copy_half(float *to, const CUtensorMap *map, int gx, int gy, uint64_t *bar) {
+__device__ __forceinline__ void tile_copy_half(void *to, const CUtensorMap *map, int gx, int gy, uint64_t *bar) {
     const int par = gy & 1;
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], "
@@ -187,26 +196,31 @@ __device__ __forceinline__ void tile_copy_half(float *to, const CUtensorMap *map
         : "memory");
 }
 
-// FP16: the region's cells on the lattice, four at a time, as their FP32 images
-// (columns [c0, c1) of the region, multiples of 4; no row wraps).
-template <int TQ, int RX, int RY, int T, typename PA>
-__device__ __forceinline__ void tile_load_f16(const PA &pl, const Geom &g, float *pop, int gx0, int gy0, int c0,
-                                              int c1) {
+// FP16: the two halves as copied to the start of `pop`, whose first cell lies
+// `shift` cells (0 or 4) before the region's, to their FP32 images in place:
+// every thread holds its cells in registers while all are read.
+template <int TQ, int RX, int RY, int T>
+__device__ __forceinline__ void tile_expand(float *pop, int shift) {
     using Lay = TileLayout<TQ, RX, RY>;
-    for (int c = (int)threadIdx.x; c < RX / 4 * RY; c += T) {
-        const int row = c / (RX / 4), x = (c - row * (RX / 4)) * 4;
-        const int gy = gy0 + row;
-        if (gy < 0 || gy >= g.ny || x < c0 || x >= c1) continue;
-        const unsigned o = (unsigned)(gy * g.pitch + gx0 + x);
-        float *const to = pop + Lay::at(row & 1, row >> 1, x);
-        float v[Lay::NQ][4];
+    constexpr int ROW = Lay::kHalfCols / 4, U = Lay::NQ * (RY / 2) * ROW, ROUNDS = (2 * U + T - 1) / T;
+    uint2 v[ROUNDS];
 #pragma unroll
-        for (int q = 0; q < Lay::NQ; ++q) {
-            const __half *p = pl.src_at(q) + o;
-            if (NOMRT_OK(g, p, 8, 61)) Ld<__half, true>::four(p, v[q]);
-        }
+    for (int k = 0; k < ROUNDS; ++k) {
+        const int n = (int)threadIdx.x + k * T, par = n >= U;
+        if (n < 2 * U)
+            v[k] = *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(pop) + par * Lay::kHalfStride +
+                                                    (n - par * U) * 8);
+    }
+    __syncthreads();
 #pragma unroll
-        for (int q = 0; q < Lay::NQ; ++q) Vec4<float>::st(to + q * Lay::PS, v[q]);
+    for (int k = 0; k < ROUNDS; ++k) {
+        const int n = (int)threadIdx.x + k * T, par = n >= U;
+        const int row = (n - par * U) / ROW, x = (n - par * U - row * ROW) * 4 - shift;
+        if (n >= 2 * U || x < 0 || x >= RX) continue;
+        __half2 h[2];
+        memcpy(h, &v[k], 8);
+        const float2 a = __half22float2(h[0]), b = __half22float2(h[1]);
+        *reinterpret_cast<float4 *>(pop + par * Lay::HS + row * RX + x) = make_float4(a.x, a.y, b.x, b.y);
     }
 }
 
@@ -421,7 +435,7 @@ template <int RY>
 __host__ __device__ constexpr int tile_rows(int k) { return RY - 2 * k; }
 
 // k steps of the tile whose first output cell is (ox, oy), ox a multiple of 4.
-// map: the source buffer's tensor map (FP32). early: read what does not change
+// map: the source buffer's tensor map. early: read what does not change
 // between steps before waiting for the previous launch (a grid whose blocks can
 // become resident before it ends).
 template <typename S, int TQ, bool BGK, int RX, int RY, int T, typename PA>
@@ -436,8 +450,11 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     uint8_t *const maps = reinterpret_cast<uint8_t *>(wall_tab + (kTileWalls + 1) * kTileWallWords);
     const int gx0 = ox - tile_margin(k), gy0 = oy - k;
     const TileWall W{wall_tab, walls.moving != 0};
-    // every region but one that wraps along y is copied in whole rows: FP32 through the tensor map
-    const bool rows = !(g.py && (gy0 < 0 || gy0 + RY > g.ny)), boxed = sizeof(S) == 4 && rows;
+    // every region but one that wraps along y is copied through the tensor map (a copy starts on 16 bytes)
+    const bool boxed = !(g.py && (gy0 < 0 || gy0 + RY > g.ny));
+    constexpr bool HALF = sizeof(S) == 2;
+    static_assert(!HALF || RX % 8 == 0, "a box row is whole 16-byte pieces");
+    const int bx0 = HALF ? gx0 & ~7 : gx0;
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
         mbar_fence_init();
@@ -461,30 +478,32 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (boxed) {
         if (threadIdx.x == 0) {
+            constexpr int BX = HALF ? Lay::kHalfCols : RX;
             // bounds-checking build: the box's first and last cells on the lattice
-            const int xa = max(gx0, 0), xb = min(gx0 + RX, g.pitch) - 1;
+            const int xa = max(bx0, 0), xb = min(bx0 + BX, g.pitch) - 1;
             const int ya = max(gy0, 0), yb = min(gy0 + RY, g.ny) - 1;
             const bool ok = NOMRT_OK(g, pl.src_at(0) + (size_t)ya * g.pitch + xa, sizeof(S), 61) &&
                             NOMRT_OK(g, pl.src_at(Lay::NQ - 1) + (size_t)yb * g.pitch + xb, sizeof(S), 61);
-            mbar_arrive_expect_tx(bar, ok ? 2u * Lay::NQ * Lay::PS * 4u : 0u);
+            mbar_arrive_expect_tx(bar, ok ? (uint32_t)(Lay::NQ * RY * BX * sizeof(S)) : 0u);
             if (ok) {
-                tile_copy_half(pop, map, gx0, gy0, bar);
-                tile_copy_half(pop + Lay::HS, map, gx0, gy0 + 1, bar);
+                tile_copy_half(pop, map, bx0, gy0, bar);
+                tile_copy_half(reinterpret_cast<char *>(pop) + (HALF ? Lay::kHalfStride : 4 * Lay::HS), map, bx0,
+                               gy0 + 1, bar);
             }
         }
-    } else if (rows) {
-        if constexpr (sizeof(S) == 2)
-            tile_load_f16<TQ, RX, RY, T>(pl, g, pop, gx0, gy0, max(0, -gx0),
-                                         (g.px ? g.nx & ~3 : g.pitch) - gx0);
     } else {
         tile_load_cells<S, TQ, RX, RY, T>(pl, g, pop, gx0, gy0, 0, RX);
     }
     if (!early) any = tile_maps<TQ, RX, RY, T>(g, maps, gx0, gy0);
     const bool walled = __syncthreads_or(any);  // also: the barrier is initialised
     if (boxed && !mbar_wait_bounded(bar, 0)) *gave_up = 1;
+    if (HALF && boxed) {
+        tile_expand<TQ, RX, RY, T>(pop, gx0 - bx0);
+        __syncthreads();
+    }
     // a periodic x: the columns beyond the seam
     const int c1 = (g.nx & ~3) - gx0;
-    if (rows && g.px && (gx0 < 0 || c1 < RX)) {
+    if (boxed && g.px && (gx0 < 0 || c1 < RX)) {
         tile_load_cells<S, TQ, RX, RY, T>(pl, g, pop, gx0, gy0, 0, min(RX, max(0, -gx0)));
         tile_load_cells<S, TQ, RX, RY, T>(pl, g, pop, gx0, gy0, max(0, min(RX, c1)), RX);
         __syncthreads();

@@ -37,7 +37,7 @@ __host__ __device__ __forceinline__ void apply_member(RatesC<float> &r, const Me
 }
 
 // One member in a launch's parameter block.
-struct alignas(64) TileMember {
+struct TileMember {
     CUtensorMap map;    // of the source buffer
     Geom g;
     const void *src;    // plane 0 of the source and of the destination buffer
@@ -109,7 +109,7 @@ struct TileBatchSet<S, ShapeOf<RX, RY, T, MINB>...> {
     static constexpr int N = sizeof...(RX);
     using One = TileSet<S, 5, false, ShapeOf<RX, RY, T, MINB>...>;
     static TilePlan plan(const KParams *const *members, int n, int sms) {
-        return choose_tile(members, n, 14, (int)sizeof(S), One::shapes(), N, sms);
+        return choose_tile(members, n, true, 14, (int)sizeof(S), One::shapes(), N, sms);
     }
     static cudaError_t maps(const KParams &p, int shape, CUtensorMap map[2]) { return One::maps(p, shape, map); }
     static cudaError_t launch(TileGroup &G, int shape, int k, cudaStream_t st) {

@@ -5,7 +5,7 @@ namespace nomrt {
 
 const TileBatchLaunchers *tile_batch_f16() {
     return TileBatchSet<__half, ShapeOf<24, 20, 224, 4>, ShapeOf<32, 20, 288, 4>, ShapeOf<32, 24, 384, 2>,
-                        ShapeOf<40, 24, 256, 4>, ShapeOf<40, 24, 128, 4>, ShapeOf<40, 32, 192, 3>>::get();
+                        ShapeOf<40, 24, 256, 4>, ShapeOf<40, 24, 128, 4>, ShapeOf<40, 32, 256, 3>>::get();
 }
 
 }  // namespace nomrt

@@ -5,7 +5,8 @@ namespace nomrt {
 
 const TileLaunchers *tile_f16_bgk() {
     return TileSet<__half, 5, true, ShapeOf<24, 20, 224, 4>, ShapeOf<32, 20, 288, 4>, ShapeOf<32, 24, 384, 2>,
-                   ShapeOf<40, 24, 256, 3>, ShapeOf<40, 24, 128, 4>, ShapeOf<48, 32, 768, 1>>::get();
+                   ShapeOf<40, 24, 256, 3>, ShapeOf<40, 24, 128, 4>, ShapeOf<40, 32, 256, 3>,
+                   ShapeOf<48, 32, 768, 1>>::get();
 }
 
 }  // namespace nomrt

@@ -69,15 +69,25 @@ inline double tile_cycles(const TileShape &s, int k, long long tiles, int nq, do
 }
 
 constexpr int kTileMaxSteps = 8;
-constexpr long long kTileMostF16 = 600000;  // cells
-constexpr double kL2Bytes = 100e6;          // what of the 129 MB L2 two buffers can count on
+constexpr double kL2Bytes = 100e6;  // what of the 129 MB L2 two buffers can count on
+
+// Cells up to which one FP16 lattice takes several steps per launch. A block
+// keeps FP32 images, so it computes as long as an FP32 lattice's and rounds
+// every population besides, while single steps are bound by HBM at half the
+// bytes. Measured, us per step, single -> several steps per launch: 1024^2 14.1
+// -> 12.0, 2048 x 1024 24.5 -> 20.2, 2500^2 59.8 -> 57.5, 4096 x 2048 72.6 ->
+// 74.3; with nine temperature populations 1777^2 49.3 -> 43.5, 4096 x 1024 53.9
+// -> 55.1. A batch's single steps are further from that bound (64 lattices of
+// 300^2: 120 -> 76) and have no such limit.
+inline double tile_most_f16(int nq) { return nq <= 14 ? 6.5e6 : 4.0e6; }
 
 // The shape and steps per launch with the least estimated time per step.
 // Lattices with node-based walls or more walls than a block keeps step once per
-// launch; so do FP16 lattices whose single steps are bound by HBM (1024^2 cells:
-// 14.0 us a step against 17.4; 600^2: 9.1 against 7.9), where the FP32 images a
-// block keeps cost more than the passes over memory they save.
-inline TilePlan choose_tile(const KParams *const *lats, int n, int nq, int elem, const TileShape *shapes,
+// launch. FP16: several regions of 32 rows per SM only where they make more than
+// two waves; below, the estimate misjudges them (600^2: 6.1 us a step against
+// 5.7; 256^2 with nine temperature populations 3.3 against 3.0; but 1111 x 333
+// 7.8 against 8.2).
+inline TilePlan choose_tile(const KParams *const *lats, int n, bool batch, int nq, int elem, const TileShape *shapes,
                             int n_shapes, int sms) {
     TilePlan best{-1, 0};
     double least = 0, cells = 0;
@@ -85,10 +95,10 @@ inline TilePlan choose_tile(const KParams *const *lats, int n, int nq, int elem,
     for (int m = 0; m < n; ++m) {
         const KParams &p = *lats[m];
         const TileCover c = tile_cover(p);
-        if (p.n_nee > 0 || p.n_walls > kTileWalls || (n == 1 && (c.rows <= 0 || c.cols <= 0))) return best;
+        if (p.n_nee > 0 || p.n_walls > kTileWalls || (!batch && (c.rows <= 0 || c.cols <= 0))) return best;
         cells += (double)p.nx * p.ny;
     }
-    if (elem == 2 && cells > kTileMostF16) return best;
+    if (elem == 2 && !batch && cells > tile_most_f16(nq)) return best;
     const double cell_bytes = 2.0 * nq * elem;
     const bool fits_l2 = cell_bytes * cells < kL2Bytes;
     for (int i = 0; i < n_shapes; ++i)
@@ -101,10 +111,12 @@ inline TilePlan choose_tile(const KParams *const *lats, int n, int nq, int elem,
                 const TileCover c = tile_cover(*lats[m]);
                 if (c.rows <= 0 || c.cols <= 0) continue;
                 const long long gx = (c.cols + tx - 1) / tx, gy = (c.rows + ty - 1) / ty;
-                fits = fits && (n > 1 || gy <= 65535);  // a lattice alone: the launch grid's y limit
+                fits = fits && (batch || gy <= 65535);  // a lattice alone: the launch grid's y limit
                 tiles += gx * gy;
             }
             if (!fits || tiles > 0x3FFFFFFF) continue;
+            if (elem == 2 && shapes[i].ry >= 32 && shapes[i].per_sm > 1 && tiles <= 2LL * sms * shapes[i].per_sm)
+                continue;
             const double t = tile_cycles(shapes[i], k, tiles, nq, cell_bytes, fits_l2, sms) / k;
             if (best.shape < 0 || t < least) {
                 best = TilePlan{i, k};
@@ -114,10 +126,10 @@ inline TilePlan choose_tile(const KParams *const *lats, int n, int nq, int elem,
     return best;
 }
 
-// The tensor map of buffer `buf` for regions of RX x RY cells: x, row pair, row
+// The tensor map of buffer `buf` for boxes of `cols` x RY cells: x, row pair, row
 // parity, plane (for an odd ny the last row pair's second row lies past the
 // plane, in the lattice's block; the kernel treats it as off the lattice).
-inline cudaError_t make_tile_map(const KParams &p, int buf, int nq, int rx, int ry, CUtensorMap *map) {
+inline cudaError_t make_tile_map(const KParams &p, int buf, int elem, int nq, int cols, int ry, CUtensorMap *map) {
     using Encode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -131,14 +143,15 @@ inline cudaError_t make_tile_map(const KParams &p, int buf, int nq, int rx, int 
         if (found != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
         entry.store(fn, std::memory_order_release);
     }
-    const cuuint64_t row = (cuuint64_t)p.pitch * 4;
+    const cuuint64_t row = (cuuint64_t)p.pitch * elem;
     const cuuint64_t dims[4] = {(cuuint64_t)p.pitch, (cuuint64_t)(p.ny + 1) / 2, 2, (cuuint64_t)nq};
-    const cuuint64_t strides[3] = {2 * row, row, (cuuint64_t)p.plane * 4};
-    const cuuint32_t box[4] = {(cuuint32_t)rx, (cuuint32_t)ry / 2, 1, (cuuint32_t)nq};
+    const cuuint64_t strides[3] = {2 * row, row, (cuuint64_t)p.plane * elem};
+    const cuuint32_t box[4] = {(cuuint32_t)cols, (cuuint32_t)ry / 2, 1, (cuuint32_t)nq};
     const cuuint32_t one[4] = {1, 1, 1, 1};
-    const CUresult r = reinterpret_cast<Encode>(fn)(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, p.pop[buf], dims, strides,
-                                                    box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+    const CUtensorMapDataType type = elem == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+    const CUresult r = reinterpret_cast<Encode>(fn)(map, type, 4, p.pop[buf], dims, strides, box, one,
+                                                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -230,13 +243,13 @@ struct TileSet<S, TQ, BGK, ShapeOf<RX, RY, T, MINB>...> {
     }
     static TilePlan plan(const KParams &p, int sms) {
         const KParams *const one = &p;
-        return choose_tile(&one, 1, 9 + TQ, (int)sizeof(S), shapes(), N, sms);
+        return choose_tile(&one, 1, false, 9 + TQ, (int)sizeof(S), shapes(), N, sms);
     }
     static cudaError_t maps(const KParams &p, int shape, CUtensorMap map[2]) {
         if (shape < 0 || shape >= N) return cudaErrorInvalidValue;
-        if (sizeof(S) != 4) return cudaSuccess;  // FP16 regions are not copied through a tensor map
         for (int b = 0; b < 2; ++b) {
-            const cudaError_t e = make_tile_map(p, b, 9 + TQ, shapes()[shape].rx, shapes()[shape].ry, map + b);
+            const cudaError_t e = make_tile_map(p, b, (int)sizeof(S), 9 + TQ, shapes()[shape].rx + (sizeof(S) == 2 ? 8 : 0),
+                                                shapes()[shape].ry, map + b);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;

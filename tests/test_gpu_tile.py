@@ -91,3 +91,48 @@ def test_runs_inside_a_callers_capture():
     side.synchronize()
     for u, v in zip(a.populations(), b.populations()):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("model", ["mrt", "q9"])
+@pytest.mark.parametrize("name", ["cavity", "box"])
+def test_lattices_of_several_waves_of_tiles(name, model, storage):
+    """Sizes that take the shapes for many tiles, the last ones ragged."""
+    import paper_1510_08224_gb300 as P
+    case = MODELS[model](lc.cavity(n=1031, Ra=1e6, n_y=909, noise=1e-3) if name == "cavity" else
+                         lc.periodic_box(1021, 903, nu=0.03, alpha=0.04, g_beta=1e-4, T0=0.5, ax=1e-5))
+    f0, g0 = lc.random_state(case, seed=5)
+    a, b = P.Lattice(case, storage=storage), P.Lattice(case, storage=storage)
+    b.set_step_kernel("scalar")
+    for lat in (a, b):
+        lat.set_populations(f0, g0)
+        lat.step(11)
+    for u, v in zip(a.populations(), b.populations()):
+        assert np.array_equal(u, v), float(np.abs(u - v).max())
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+def test_batch_runs_equal_single_steps_alone(storage):
+    """Members whose tiles are ragged, wrap, or have moving and many walls, more
+    than one launch takes, joined at odd and even steps."""
+    import paper_1510_08224_gb300 as P
+    names = ["cavity_20x13", "rb_3x40", "couette_5x9", "solids_261x19", "box_1x1", "rb_133x7", "walls_15"]
+    cases = [CASES[names[i % len(names)]] for i in range(69)] + [lc.cavity(n=301, Ra=1e5, n_y=203, noise=1e-3)]
+    a = [P.Lattice(c, storage=storage) for c in cases]
+    b = [P.Lattice(c, storage=storage) for c in cases]
+    batch = P.Batch()
+    for i, (case, u, v) in enumerate(zip(cases, a, b)):
+        f0, g0 = lc.random_state(case, seed=i)
+        v.set_step_kernel("scalar")
+        for lat in (u, v):
+            lat.set_populations(f0, g0)
+            lat.step(i % 3)
+        batch.add(u)
+    for n in (2, 3, 16):
+        batch.step(n)
+        for lat in b:
+            lat.step(n)
+        for u, v in zip(a, b):
+            for x, y in zip(u.populations(), v.populations()):
+                assert np.array_equal(x, y), n
+    batch.close()
