@@ -5,7 +5,7 @@ Workload: Rayleigh-Benard cell, 4096 x 2048 fluid cells (plus the two wall
 rows), periodic in x, Ra = 1e6, Pr = 0.71, Ma = 0.1, seeded 1e-3 Gaussian
 temperature perturbation; FP32-shifted population storage by default.
 
-One bench step = one time step of the whole lattice (one fused kernel launch).
+One bench step = one time step of the whole lattice (a launch takes up to eight).
 value = fluid cells x steps / time / 1e6 (MLUPS), timed with CUDA events on the
 lattice's stream, inputs resident in HBM. The working set (two population
 buffers, > 1 GB) is far larger than L2, so no flush is needed between steps.
@@ -48,7 +48,8 @@ def workload(nx: int, H: int):
 # launched: the kernel translation units and every header they include (host
 # code such as the batch executor or the C-ABI entry points is not part of it).
 STEP_KERNEL_SOURCES = ("kernels_f64.cu", "kernels_f32.cu", "kernels_f16.cu", "launchers.cuh", "nomrt_kernels.cuh",
-                       "nomrt_internal.h", "step8.cuh", "step_tma.cuh")
+                       "nomrt_internal.h", "step8.cuh", "step_tma.cuh", "tile.cuh", "tile_launch.cuh", "tile_f32.cu",
+                       "tile_f16.cu")
 
 
 def kernel_source_hash() -> str:
@@ -90,12 +91,13 @@ def profile_values(name: str):
     return vals
 
 
-def profiled_traffic(storage: str, nx: int, ny: int):
+def profiled_traffic(storage: str, nx: int, ny: int, steps_per_launch: int):
     """DRAM bytes per step-kernel launch from the committed ncu summary, or None
     if there is none for this storage and size, or the kernel sources changed
     since it was taken."""
+    kernel = "step" if steps_per_launch == 1 else "tile"
     try:
-        return float(profile_values(f"k_step_{storage}_rb{nx}x{ny - 2}.md")["traffic_bytes_per_launch"])
+        return float(profile_values(f"k_{kernel}_{storage}_rb{nx}x{ny - 2}.md")["traffic_bytes_per_launch"])
     except (KeyError, ValueError):
         return None
 
@@ -447,6 +449,8 @@ def run_batched(args):
               flush=True)
         return 0
     tuned_kind, tuned_cfg, ms_cand = b.tune(trial_steps=64)
+    if tuned_kind == "fused" and b.steps_per_launch() > 1:
+        tuned_cfg = -1  # several steps per launch
     tuned_unit = b.info()["rows_per_unit"]
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
@@ -480,7 +484,7 @@ def run_batched(args):
             set_member_kernel(b, cfg)
         elif kind == "fused":
             cands = {c: ms_cand[f"fused_cfg{c}"] for c in range(10)}
-            cfg = min(cands, key=cands.get)
+            cfg = -1 if tuned_kind == "fused" and tuned_cfg < 0 else min(cands, key=cands.get)
             b.set_config(cfg, 1)
         else:
             cands = {(c, 1): ms_cand[f"persistent_cfg{c}"] for c in range(5)}
@@ -506,7 +510,10 @@ def run_batched(args):
     ms = timed(b.step, args.steps)
     t_end = time.perf_counter()
     sampler.stop()
-    launches_per_step = {"fused": 1, "persistent": 1 / 32, "concurrent": args.count}[tuned_kind]
+    per_launch = b.steps_per_launch()
+    graph_launches = -(-32 // per_launch)  # per graph of 32 steps: an even number
+    graph_launches += graph_launches & 1 if tuned_cfg < 0 else 0
+    launches_per_step = {"fused": graph_launches / 32, "persistent": 1 / 32, "concurrent": args.count}[tuned_kind]
     finite = True
     for lat in lats:
         try:
@@ -523,7 +530,9 @@ def run_batched(args):
     ms_serial = timed(serial, k_serial)
     tuned = rate(ms, args.steps)
     value = tuned["MLUPS"]
-    kernel = {"fused": "k_batch_grid_w" if tuned_cfg >= 5 else "k_batch_grid", "persistent": "k_batch_persistent",
+    # a launch of several steps reads and writes every population once
+    hbm = tuned["frac"] * (launches_per_step if tuned_kind == "fused" else 1)
+    kernel = {"fused": "k_batch_grid_w" if tuned_cfg >= 5 else "k_batch_grid" if tuned_cfg >= 0 else "k_tile_batch", "persistent": "k_batch_persistent",
               "concurrent": "each member's step kernel, concurrent streams"}[tuned_kind]
     line = {
         "metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": 1, "steps": args.steps,
@@ -535,14 +544,16 @@ def run_batched(args):
                    "storage": STORAGE_NAME[args.storage],
                    "tuned": {"kind": tuned_kind, "config": tuned_cfg, "member_kernel": member_kernel,
                              "rows_per_unit": tuned_unit if tuned_kind == "persistent" else None, "graph_steps": 32,
-                             "steps_per_launch": 32 if tuned_kind == "persistent" else 1},
+                             "steps_per_launch": per_launch},
                    "l2": "no flush: working set > L2",
                    "tune_ms_per_step": {k: (round(m, 5) if np.isfinite(m) else None) for k, m in ms_cand.items()}},
         "kinds": kinds,
         "finite": finite,
         "serial_per_lattice": {**rate(ms_serial, k_serial), "steps": k_serial, "launches_per_step": args.count},
-        "roofline": {"bound": "hbm", "achieved": round(bpn * cells / (tuned["ms_per_step"] * 1e-3) / 1e9, 1),
-                     "peak": peak, "unit": "GB/s", "frac": tuned["frac"], "traffic": None, "kernel": kernel,
+        "roofline": {"bound": "hbm" if tuned_cfg >= 0 or tuned_kind != "fused" else
+                     "shared-memory and FP32 pipes (HBM share given)",
+                     "achieved": round(hbm * peak, 1), "peak": peak, "unit": "GB/s", "frac": round(hbm, 4),
+                     "traffic": None, "kernel": kernel,
                      "bytes_per_node": bpn, "peak_source": f"{peak_src} HBM copy bandwidth (burst)"},
         "gpu_launches": int(round(args.steps * launches_per_step)),
         "clocks": sampler.summary(t_start, t_end),
@@ -879,6 +890,8 @@ def main():
     ms_max = reduce_max_time(ms, dist, "cuda")
     sampler.stop()
     clocks = sampler.summary(t_start, t_end)
+    per_launch = lat.steps_per_launch() if args.steps > 1 else 1
+    launches = -(-args.steps // per_launch)
     r = lat.residual()  # residual over the timed steps: finite, or LBMError if the state diverged
     lat.close()
     del lat
@@ -886,11 +899,15 @@ def main():
     value = whole_job_mlups(fluid, args.steps, world, ms_max)
     ms_step = ms_max / args.steps
     peak, peak_src = measured_peak()
-    achieved = BYTES_PER_NODE[args.storage] * fluid / (ms / args.steps * 1e-3) / 1e9
-    traffic = profiled_traffic(args.storage, args.nx, args.H + 2)
-    roof = {"bound": "hbm" if args.storage != "f64" else "alu", "achieved": round(achieved, 1),
+    # a launch reads and writes every population once, however many steps it takes
+    achieved = BYTES_PER_NODE[args.storage] * fluid * launches / (ms * 1e-3) / 1e9
+    traffic = profiled_traffic(args.storage, args.nx, args.H + 2, per_launch)
+    roof = {"bound": "alu" if args.storage == "f64" else "hbm" if per_launch == 1 else
+            "shared-memory and FP32 pipes (HBM share given)", "achieved": round(achieved, 1),
             "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4), "traffic": traffic,
-            "kernel": "k_step", "bytes_per_node": BYTES_PER_NODE[args.storage],
+            "kernel": "k_step" if per_launch == 1 else "k_tile", "steps_per_launch": per_launch,
+            "one_pass_per_step_frac": round(achieved / peak * args.steps / launches, 4),
+            "bytes_per_node": BYTES_PER_NODE[args.storage],
             "peak_source": f"{peak_src} HBM copy bandwidth (burst)"}
     dfma = None
     if args.storage == "f64" or not args.no_variants:
@@ -915,7 +932,7 @@ def main():
                          f"{BYTES_PER_NODE[args.storage] // 2 * fluid / 1e9:.2f} GB each)",
                    "parallelism": f"replicas{world}", "step_kernel": [args.variant, args.config]},
         "roofline": roof,
-        "gpu_launches": args.steps,
+        "gpu_launches": launches,
         "clocks": clocks,
         "residual_check": r,
     }
@@ -937,8 +954,9 @@ def main():
                 continue
             k = max(10, min(args.steps, 500))
             vms, vl = time_steps(P, torch, case, st, k, args.warmup)
+            per = vl.steps_per_launch()
             vl.close()
-            vach = BYTES_PER_NODE[st] * fluid / (vms / k * 1e-3) / 1e9
+            vach = BYTES_PER_NODE[st] * fluid * -(-k // per) / (vms * 1e-3) / 1e9
             vm = fluid * k / (vms * 1e-3) / 1e6
             var[STORAGE_NAME[st]] = {"MLUPS": round(vm, 1), "steps": k,
                                      "GB/s": round(vach, 1), "frac": round(vach / peak, 4)}

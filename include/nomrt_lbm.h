@@ -163,7 +163,7 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
 /* Advance nsteps >= 0 time steps (Eqs. 8-9 and 24-25, fused). Asynchronous on the
  * lattice's stream. With the AUTO step kernel, runs of two steps or more of an
  * FP32 or FP16 lattice without node-based walls (and with at most 15 walls; in
- * FP16 up to 600,000 cells) take up to eight steps per launch, tile by tile in
+ * FP16 up to 6.5 million cells, 4 million with nine temperature populations) take up to eight steps per launch, tile by tile in
  * shared memory, the tile and the steps per launch chosen from the lattice's
  * size; the bits are those of single steps. Every other step is one kernel,
  * plus one for the boundary nodes of node-based walls; runs of 4 such steps or
@@ -173,6 +173,9 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
  * shorter runs and the remainder, and calls on a stream that is being captured,
  * launch the kernels directly. */
 lbm_status lbm_step(lbm_lattice *h, int64_t nsteps);
+
+/* The most steps a launch of lbm_step takes for h with its step kernel: 1 to 8. */
+lbm_status lbm_steps_per_launch(lbm_lattice *h, int32_t *steps);
 
 /* Wait for the lattice's stream. LBM_ETIMEOUT if a step kernel gave up one of
  * its bounded waits since the last check (the state is then undefined). */
@@ -338,9 +341,12 @@ lbm_status lbm_batch_add(lbm_batch *b, lbm_lattice *h);
 lbm_status lbm_batch_remove(lbm_batch *b, lbm_lattice *h);
 
 /* How a batch step runs.
- * FUSED (the default): one kernel launch per step and launch group, one
- * 128-thread block of the four-cell row code per 512-cell row segment of every
- * member (a 1-D grid over the members' segments).
+ * FUSED (the default): one kernel launch per launch group for up to eight
+ * steps, each block updating one tile of a member in shared memory; where a
+ * member has node-based walls or more than 15 walls, or a config is set, one
+ * launch per step, one 128-thread block of the four-cell row code per 512-cell
+ * row segment of every member (a 1-D grid over the members' segments). The bits
+ * are the same.
  * PERSISTENT: one cooperative launch per group for steps_per_launch steps: its
  * resident blocks stride over the same row segments, with a clock-bounded grid
  * barrier between steps (LBM_ETIMEOUT from lbm_batch_sync if one expires). A
@@ -364,8 +370,9 @@ lbm_status lbm_batch_set_mode(lbm_batch *b, int32_t steps_per_launch, int32_t gr
 lbm_status lbm_batch_get_mode(const lbm_batch *b, int32_t *kind, int32_t *steps_per_launch, int32_t *graph_steps);
 
 /* Kernel shape of the FUSED and PERSISTENT kinds: config 0..4 asks ptxas for
- * 4..8 resident 128-thread blocks per SM (-1: the default, 6 for FP32 and 3 for
- * FP16), one block per 512-cell row segment; config 5..9, for the FUSED kind,
+ * 4..8 resident 128-thread blocks per SM, one block per 512-cell row segment
+ * (-1, the default: several steps per launch in the FUSED kind, else 6 for FP32
+ * and 3 for FP16); config 5..9, for the FUSED kind,
  * the same occupancies with one 128-cell row segment per warp (four per
  * block), so that rows that are not a multiple of 512 cells leave no warp of a
  * block idle (the PERSISTENT kind runs config c as c - 5); rows_per_unit
@@ -399,13 +406,19 @@ lbm_status lbm_batch_get_member_kernel(const lbm_batch *b, int32_t *variant, int
  * step of every candidate in ms_per_step[31] (FUSED 0-9, PERSISTENT 0-4 with
  * one-segment units, PERSISTENT 0-4 with two-segment units, CONCURRENT own,
  * CONCURRENT VEC4 0-4, CONCURRENT VEC4W 0-4; +inf for a
- * candidate that cannot run, such as PERSISTENT with node-based walls). Any
+ * candidate that cannot run, such as PERSISTENT with node-based walls). The
+ * FUSED kind's several steps per launch are timed too and, where fastest, kept
+ * (config -1; *best_config then holds the config of its single steps). Any
  * output may be NULL. Synchronises. */
 lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *best_kind, int32_t *best_config,
                           float *ms_per_step);
 
 /* Advance every member by nsteps (asynchronous on the batch's stream). */
 lbm_status lbm_batch_step(lbm_batch *b, int64_t nsteps);
+
+/* The most steps a launch of lbm_batch_step takes with the kind, mode, config
+ * and members in force. */
+lbm_status lbm_batch_steps_per_launch(lbm_batch *b, int32_t *steps);
 
 /* Wait for the batch's stream; LBM_ETIMEOUT if a persistent launch gave up a
  * grid barrier (the members' state is then undefined; later persistent
@@ -422,14 +435,13 @@ lbm_status lbm_batch_debug_barrier_extra(lbm_batch *b, int32_t extra);
 
 /* The steady-state residual of every member (lbm_residual's R, against and
  * then replacing each member's own snapshot; +infinity at a member's first
- * call), with one synchronisation for the whole batch: the members' residual
- * kernels run on the batch's stream, their sums land side by side and come
- * back in one copy. members[i] (may be NULL) and r[i] for i < *n, in the
+ * call), with one synchronisation for the whole batch: one kernel per 64 members
+ * on the batch's stream, which leaves the sums in page-locked host memory. members[i] (may be NULL) and r[i] for i < *n, in the
  * batch's member order; cap: the capacity of both arrays (LBM_EINVAL if
  * below the member count, *n still set). A member whose fields are not finite
  * gets r[i] = NaN (lbm_residual would return LBM_EDIVERGED for it). The batch
- * allocates its device and pinned host buffers for the sums (cudaMalloc,
- * cudaHostAlloc) when it first needs them. Synchronises. */
+ * allocates the page-locked buffer of the sums (cudaHostAlloc) when it first
+ * needs it. Synchronises. */
 lbm_status lbm_batch_residuals(lbm_batch *b, int32_t cap, lbm_lattice **members, double *r, int32_t *n);
 
 /* Members, their fluid cells, 512-cell row segments per step (summed over the

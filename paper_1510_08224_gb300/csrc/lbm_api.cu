@@ -1193,6 +1193,12 @@ lbm_status lbm_info(const lbm_lattice *h, int64_t *fluid_cells, int32_t *pitch, 
     return LBM_OK;
 }
 
+lbm_status lbm_steps_per_launch(lbm_lattice *h, int32_t *steps) {
+    if (!h || !steps) return LBM_EINVAL;
+    *steps = h->kp.variant == nomrt::kStepAuto && plan_tiles(h) ? h->tile_plan.steps : 1;
+    return LBM_OK;
+}
+
 const char *lbm_last_error(const lbm_lattice *h) {
     if (!h) return g_create_error.c_str();
     return h->err.c_str();

@@ -1267,6 +1267,16 @@ lbm_status lbm_batch_get_mode(const lbm_batch *b, int32_t *kind, int32_t *steps_
     return LBM_OK;
 }
 
+lbm_status lbm_batch_steps_per_launch(lbm_batch *b, int32_t *steps) {
+    if (!b || !steps) return LBM_EINVAL;
+    const lbm_status st = rebuild(b);
+    if (st != LBM_OK) return st;
+    *steps = 1;
+    if (b->kind == LBM_BATCH_FUSED && b->config < 0 && b->tile_plan.shape >= 0) *steps = b->tile_plan.steps;
+    else if (b->kind == LBM_BATCH_PERSISTENT && !any_nee(b)) *steps = b->steps_per_launch;
+    return LBM_OK;
+}
+
 const char *lbm_batch_last_error(const lbm_batch *b) {
     if (!b) return lbm_last_error(nullptr);
     return b->err.c_str();

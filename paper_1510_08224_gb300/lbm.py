@@ -25,11 +25,12 @@ STEP_VARIANTS = {"auto": 0, "scalar": 1, "vec4": 2, "tma": 3, "vec8": 4, "vec4w"
 EXPORTED = ("lbm_footprint_bytes", "lbm_validate", "lbm_create", "lbm_step", "lbm_sync", "lbm_step_kernel_count",
             "lbm_set_step_kernel", "lbm_read_macro", "lbm_read_macro_rows",
             "lbm_nusselt",
-            "lbm_residual", "lbm_get_populations", "lbm_set_populations", "lbm_info", "lbm_last_error",
+            "lbm_residual", "lbm_get_populations", "lbm_set_populations", "lbm_info", "lbm_steps_per_launch", "lbm_last_error",
             "lbm_destroy", "lbm_residual_fields_noalloc", "lbm_probe_fp64_rate", "lbm_bounds_checking",
             "lbm_debug_bounds_limit", "lbm_batch_create", "lbm_batch_add", "lbm_batch_remove",
             "lbm_batch_set_mode", "lbm_batch_set_kind", "lbm_batch_set_config", "lbm_batch_tune", "lbm_batch_step", "lbm_batch_sync",
-            "lbm_batch_info", "lbm_batch_get_mode", "lbm_batch_residuals", "lbm_batch_last_error", "lbm_batch_destroy",
+            "lbm_batch_info", "lbm_batch_get_mode", "lbm_batch_residuals", "lbm_batch_steps_per_launch",
+            "lbm_batch_last_error", "lbm_batch_destroy",
             "lbm_batch_debug_barrier_extra", "lbm_batch_set_member_kernel", "lbm_batch_get_member_kernel")
 BATCH_KINDS = {"fused": 0, "concurrent": 1, "persistent": 2}
 
@@ -115,6 +116,8 @@ def load():
         L.lbm_info.restype = C.c_int
         L.lbm_info.argtypes = [vp, C.POINTER(C.c_int64), C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                C.POINTER(C.c_int64)]
+        L.lbm_steps_per_launch.restype = C.c_int
+        L.lbm_steps_per_launch.argtypes = [vp, C.POINTER(C.c_int32)]
         L.lbm_last_error.restype = C.c_char_p
         L.lbm_last_error.argtypes = [vp]
         L.lbm_destroy.restype = None
@@ -127,7 +130,8 @@ def load():
                            ("lbm_batch_get_mode", [vp, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                                    C.POINTER(C.c_int32)]),
                            ("lbm_batch_residuals", [vp, C.c_int32, C.POINTER(vp), dp, C.POINTER(C.c_int32)]),
-                           ("lbm_batch_step", [vp, C.c_int64]), ("lbm_batch_sync", [vp]),
+                           ("lbm_batch_step", [vp, C.c_int64]), ("lbm_batch_steps_per_launch", [vp, C.POINTER(C.c_int32)]),
+                           ("lbm_batch_sync", [vp]),
                            ("lbm_batch_debug_barrier_extra", [vp, C.c_int32]),
                            ("lbm_batch_set_member_kernel", [vp, C.c_int32, C.c_int32]),
                            ("lbm_batch_get_member_kernel", [vp, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
@@ -363,6 +367,12 @@ class Lattice:
         _check(load().lbm_info(self._h, C.byref(fl), C.byref(pitch), C.byref(eb), C.byref(st)), self._h)
         return dict(fluid_cells=fl.value, pitch=pitch.value, elem_bytes=eb.value, steps=st.value)
 
+    def steps_per_launch(self) -> int:
+        """The most time steps one launch of step() takes (lbm_steps_per_launch)."""
+        n = C.c_int32()
+        _check(load().lbm_steps_per_launch(self._h, C.byref(n)), self._h)
+        return n.value
+
 
 class Batch:
     """Lattices of uneven size advanced together (see the lbm_batch_* calls).
@@ -408,7 +418,7 @@ class Batch:
         return names[k.value], spl.value, gs.value
 
     def set_kind(self, kind):
-        """'fused' (one launch per step over every member's rows), 'persistent'
+        """'fused' (one launch over every member for up to eight steps), 'persistent'
         (one cooperative launch per steps_per_launch steps, grid barrier between
         steps) or 'concurrent' (a single-lattice kernel per member, side by side)."""
         k = BATCH_KINDS[kind] if isinstance(kind, str) else int(kind)
@@ -431,6 +441,12 @@ class Batch:
         names = {n: k for k, n in STEP_VARIANTS.items()}
         return names[v.value], c.value
 
+    def steps_per_launch(self) -> int:
+        """The most time steps one launch takes (lbm_batch_steps_per_launch)."""
+        n = C.c_int32()
+        self._check(load().lbm_batch_steps_per_launch(self._h, C.byref(n)))
+        return n.value
+
     def tune(self, trial_steps: int = 8):
         """Autotune kind and config on the current members (state unchanged).
         Returns (kind name, config, {candidate: ms per step}) with candidates
@@ -440,7 +456,8 @@ class Batch:
         concurrent (the members' own kernels),
         concurrent_vec4_cfg0-4 and concurrent_vec4w_cfg0-4; for the concurrent
         kind the config is -1 (own), 0-4 (vec4) or 5-9 (vec4w), already in
-        force as the member kernel."""
+        force as the member kernel. The fused kind's several steps per launch
+        are timed too and, where fastest, kept (steps_per_launch() then says so)."""
         kind, cfg = C.c_int32(), C.c_int32()
         ms = (C.c_float * 31)()
         self._check(load().lbm_batch_tune(self._h, int(trial_steps), C.byref(kind), C.byref(cfg), ms))
