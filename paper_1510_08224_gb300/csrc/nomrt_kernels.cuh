@@ -895,9 +895,10 @@ __global__ void __launch_bounds__(128) k_nee(const Planes<S> pl, const Geom g, c
 
 // The FP64 step: one cell per thread in blocks of two warps, cells numbered along
 // the rows without regard to their ends (flat) or, in lattices of a few warps per
-// SM, where a step is a chain of latencies, along one row per grid row. NODES: the boundary nodes of node-based walls are the first blocks'
-// (they read the same source buffer and write cells no other thread writes). Bound by the FP64 pipe: 94 instructions
-// of 16 cycles per warp and SM. Small blocks and no idle row ends because a
+// SM, where a step is a chain of latencies, along one row per grid row. NODES:
+// the boundary nodes of node-based walls are the first blocks' (they read the
+// same source buffer and write cells no other thread writes). Bound by the FP64
+// pipe: 94 instructions of 16 cycles per warp and SM. Small blocks and no idle row ends because a
 // lattice of 256^2 cells gives an SM about 14 warps: with 128 x 2 blocks (three
 // per row pair, the third nearly empty) some SMs ran half as many again, and a
 // second launch for the nodes, 16 warps on 4 SMs, took as long as the cells.
@@ -1151,8 +1152,12 @@ __global__ void __launch_bounds__(kRedThreads) k_nusselt(const Planes<S> pl, con
 }
 
 // One block's cells of a residual over `blocks` blocks: v += |du|^2, |u|^2, dT^2,
-// T^2, non-finite cells; the snapshot takes the new values. Bound by the FP64
-// pipe on large lattices: 13 operations per cell.
+// T^2, non-finite cells; the snapshot takes the new values. On large lattices
+// the FP64 pipe (17 operations per cell, conversions included) and the loads it
+// waits for; every load of a cell in flight at once and four blocks per SM: 4096
+// x 2048 455 -> 282 us (FP16 990 -> 285). Small ones are a launch and a wait: 56
+// -> 24 us a call with the sums and status words written to the host by the last
+// block instead of a second kernel and two copies.
 template <typename S, int TQ>
 __device__ __forceinline__ void residual_cells(const S *const *src, const Geom &g,
                                                const RatesC<typename Store<S>::C> &r, double T_ref, double *snap,
