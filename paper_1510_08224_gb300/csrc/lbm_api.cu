@@ -1017,20 +1017,19 @@ lbm_status lbm_read_macro_rows(lbm_lattice *h, int32_t y0, int32_t y1, double *r
     // host memory where it shares the host's page tables; any other sends every output through the staging
     // area
     double *direct[4] = {nullptr, nullptr, nullptr, nullptr};
-    bool in_place = true, ordinary = false;
+    bool in_place = true, ordinary[4] = {};
     for (int k = 0; k < 4; ++k)
         if (outs[k]) {
             direct[k] = static_cast<double *>(const_cast<void *>(device_view(outs[k])));
             if (!direct[k] && reaches_host()) {
                 direct[k] = outs[k];
-                ordinary = true;
+                ordinary[k] = true;
             }
             in_place = in_place && direct[k];
         }
     if (in_place) {
-        if (ordinary)
-            for (int k = 0; k < 4; ++k)
-                if (outs[k] && direct[k] == outs[k]) touch_pages(outs[k], (size_t)(y1 - y0) * nx * sizeof(double));
+        for (int k = 0; k < 4; ++k)
+            if (ordinary[k]) touch_pages(outs[k], (size_t)(y1 - y0) * nx * sizeof(double));
         const bool brief = reaches_host();  // the status words come along
         h->msg.status[0] = nomrt::kStatusOk;
         h->msg.status[1] = 0;

@@ -1,0 +1,48 @@
+"""Where lbm_read_macro may write: outputs of different kinds of memory in one
+call give the values of a plain read."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+import lbm_cases as lc
+
+pytestmark = pytest.mark.gpu
+
+
+def _lattice(storage="f32"):
+    import paper_1510_08224_gb300 as P
+    case = lc.rayleigh_benard(nx=301, H=68, Ra=1e5, sigma=1e-2)
+    lat = P.Lattice(case, storage=storage)
+    lat.step(40)
+    return P, lat
+
+
+def _output(kind, ny, nx):
+    """(the object that owns ny x nx doubles of memory of a kind, their address)."""
+    import torch
+    if kind == "pageable":
+        a = np.full((ny, nx), -1.1)
+        return a, a.ctypes.data
+    t = torch.full((ny, nx), -1.1, dtype=torch.float64)
+    t = t.cuda() if kind == "device" else t.pin_memory()
+    return t, t.data_ptr()
+
+
+def _values(owner):
+    return owner if isinstance(owner, np.ndarray) else owner.cpu().numpy()
+
+
+@pytest.mark.parametrize("kinds", [("pageable", "device", "page-locked", None), ("device", None, "pageable", "pageable"),
+                                   ("page-locked", "pageable", None, "device")])
+def test_outputs_of_several_kinds_in_one_call(kinds):
+    """A pageable output beside a device or a page-locked one: the host maps the
+    pages of the pageable one alone."""
+    P, lat = _lattice()
+    ref = lat.macro()
+    outs = [None if k is None else _output(k, lat.ny, lat.nx) for k in kinds]
+    ptr = [None if o is None else C.cast(o[1], C.POINTER(C.c_double)) for o in outs]
+    assert P.load().lbm_read_macro(lat.handle, *ptr) == 0
+    for o, r in zip(outs, ref):
+        assert o is None or np.array_equal(_values(o[0]), r)
+    lat.close()
