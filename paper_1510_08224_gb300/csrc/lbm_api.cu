@@ -1014,14 +1014,15 @@ lbm_status lbm_read_macro_rows(lbm_lattice *h, int32_t y0, int32_t y1, double *r
     double *outs[4] = {rho, ux, uy, T};
     const int nx = h->nx;
     // outputs the GPU reaches are written by the kernel in place: page-locked or device ones, and ordinary
-    // host memory where it shares the host's page tables; any other sends every output through the staging
-    // area
+    // host memory where it shares the host's page tables; any other, and one that is not on a double's
+    // boundary (the kernel stores whole doubles), sends every output through the staging area
     double *direct[4] = {nullptr, nullptr, nullptr, nullptr};
     bool in_place = true, ordinary[4] = {};
     for (int k = 0; k < 4; ++k)
         if (outs[k]) {
-            direct[k] = static_cast<double *>(const_cast<void *>(device_view(outs[k])));
-            if (!direct[k] && reaches_host()) {
+            const bool aligned = (uintptr_t)outs[k] % alignof(double) == 0;
+            if (aligned) direct[k] = static_cast<double *>(const_cast<void *>(device_view(outs[k])));
+            if (aligned && !direct[k] && reaches_host()) {
                 direct[k] = outs[k];
                 ordinary[k] = true;
             }
@@ -1058,7 +1059,7 @@ lbm_status lbm_read_macro_rows(lbm_lattice *h, int32_t y0, int32_t y1, double *r
                 if (outs[k])
                     LBM_CUDA(h,
                              cudaMemcpyAsync(outs[k] + (size_t)(r0 - y0) * nx, h->stage() + k * n, n * sizeof(double),
-                                             cudaMemcpyDeviceToHost, h->stream),
+                                             cudaMemcpyDefault, h->stream),
                              "read macro");
         }
     }

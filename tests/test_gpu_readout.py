@@ -1,5 +1,5 @@
 """Where lbm_read_macro may write: outputs of different kinds of memory in one
-call give the values of a plain read."""
+call, and outputs on any byte, give the values of a plain read."""
 import ctypes as C
 
 import numpy as np
@@ -45,4 +45,28 @@ def test_outputs_of_several_kinds_in_one_call(kinds):
     assert P.load().lbm_read_macro(lat.handle, *ptr) == 0
     for o, r in zip(outs, ref):
         assert o is None or np.array_equal(_values(o[0]), r)
+    lat.close()
+
+
+@pytest.mark.parametrize("kinds", [("pageable",) * 4, ("page-locked",) * 4, ("device",) * 4,
+                                   ("pageable", None, "device", "page-locked")])
+@pytest.mark.parametrize("shift", [1, 4])
+def test_outputs_on_any_byte(kinds, shift):
+    """Outputs that are not on a double's boundary (views into packed buffers)
+    take the staging area, whatever memory they lie in."""
+    import torch
+    P, lat = _lattice()
+    ref = lat.macro()
+    n = 8 * lat.ny * lat.nx
+    outs = []
+    for kind in kinds:
+        t = torch.full((n + 8,), 7, dtype=torch.uint8, pin_memory=kind == "page-locked")
+        outs.append(None if kind is None else t.cuda() if kind == "device" else t)
+    ptr = [None if t is None else C.cast(t.data_ptr() + shift, C.POINTER(C.c_double)) for t in outs]
+    assert P.load().lbm_read_macro(lat.handle, *ptr) == 0
+    for t, r in zip(outs, ref):
+        if t is not None:
+            b = t.cpu().numpy()
+            assert np.array_equal(b[shift:shift + n].copy().view(np.float64).reshape(r.shape), r)
+            assert (b[:shift] == 7).all() and (b[shift + n:] == 7).all()
     lat.close()
