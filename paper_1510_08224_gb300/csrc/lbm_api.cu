@@ -885,11 +885,12 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
                                  cudaMemcpyHostToDevice, st)) != cudaSuccess)
             return cuda_bail(e, "upload boundary nodes");
     }
-    // initial state (and zeros in the other buffer): T read in place when the GPU can reach it
-    // (or T0 everywhere), else in row chunks through the staging area, which holds nq rows of
+    // initial state (and zeros in the other buffer): T read in place when the GPU can reach it and it lies on
+    // a double's boundary (or T0 everywhere), else in row chunks through the staging area, which holds nq rows of
     // populations and so stage_rows * nq rows of T. Stream order keeps a chunk's upload behind
     // the previous chunk's init kernel; one wait at the end covers the host buffers.
-    const double *Tv = p->T_init ? static_cast<const double *>(device_view(p->T_init)) : nullptr;
+    const bool T_aligned = (uintptr_t)p->T_init % alignof(double) == 0;
+    const double *Tv = p->T_init && T_aligned ? static_cast<const double *>(device_view(p->T_init)) : nullptr;
     if (!p->T_init || Tv) {
         for (int r0 = 0; r0 < ny; r0 += 65535) {
             const int r1 = std::min(ny, r0 + 65535);
@@ -902,7 +903,7 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
         for (int r0 = 0; r0 < ny; r0 += t_rows) {
             const int r1 = std::min(ny, r0 + t_rows);
             if ((e = cudaMemcpyAsync(h->stage(), p->T_init + (size_t)r0 * nx, (size_t)(r1 - r0) * nx * sizeof(double),
-                                     cudaMemcpyHostToDevice, st)) != cudaSuccess)
+                                     cudaMemcpyDefault, st)) != cudaSuccess)
                 return cuda_bail(e, "upload T_init");
             if ((e = h->L->init_rows(kp, 0, r0, r1, h->stage(), st)) != cudaSuccess)
                 return cuda_bail(e, "init kernel");

@@ -1,5 +1,6 @@
 """Where lbm_read_macro may write: outputs of different kinds of memory in one
-call, and outputs on any byte, give the values of a plain read."""
+call, and outputs on any byte, give the values of a plain read; and lbm_create
+takes its initial temperature from any byte."""
 import ctypes as C
 
 import numpy as np
@@ -70,3 +71,26 @@ def test_outputs_on_any_byte(kinds, shift):
             assert np.array_equal(b[shift:shift + n].copy().view(np.float64).reshape(r.shape), r)
             assert (b[:shift] == 7).all() and (b[shift + n:] == 7).all()
     lat.close()
+
+
+@pytest.mark.parametrize("kind", ["pageable", "page-locked", "device"])
+def test_initial_temperature_on_any_byte(kind):
+    """A T_init that is not on a double's boundary is staged, not read in place."""
+    import torch
+    P, lat = _lattice()
+    case = lat.case
+    n = 8 * case.ny * case.nx
+    t = torch.zeros(n + 8, dtype=torch.uint8, pin_memory=kind == "page-locked")
+    t.numpy()[3:3 + n] = np.ascontiguousarray(case.T_init, dtype=np.float64).reshape(-1).view(np.uint8)
+    t = t.cuda() if kind == "device" else t
+    p, keep = P.make_params(case, "f32")
+    p.T_init = t.data_ptr() + 3
+    h = C.c_void_p()
+    L = P.load()
+    assert L.lbm_create(C.byref(p), None, None, C.c_size_t(0), C.byref(h)) == 0
+    T = np.zeros((case.ny, case.nx))
+    assert L.lbm_read_macro(h, None, None, None, C.cast(T.ctypes.data, C.POINTER(C.c_double))) == 0
+    assert np.array_equal(T, P.Lattice(case, storage="f32").macro()[3])
+    L.lbm_destroy(h)
+    lat.close()
+    del keep
