@@ -2,6 +2,8 @@
 call, and outputs on any byte, give the values of a plain read; and lbm_create
 takes its initial temperature from any byte."""
 import ctypes as C
+import threading
+import time
 
 import numpy as np
 import pytest
@@ -11,9 +13,9 @@ import lbm_cases as lc
 pytestmark = pytest.mark.gpu
 
 
-def _lattice(storage="f32"):
+def _lattice(storage="f32", nx=301, H=68):
     import paper_1510_08224_gb300 as P
-    case = lc.rayleigh_benard(nx=301, H=68, Ra=1e5, sigma=1e-2)
+    case = lc.rayleigh_benard(nx=nx, H=H, Ra=1e5, sigma=1e-2)
     lat = P.Lattice(case, storage=storage)
     lat.step(40)
     return P, lat
@@ -37,8 +39,8 @@ def _values(owner):
 @pytest.mark.parametrize("kinds", [("pageable", "device", "page-locked", None), ("device", None, "pageable", "pageable"),
                                    ("page-locked", "pageable", None, "device")])
 def test_outputs_of_several_kinds_in_one_call(kinds):
-    """A pageable output beside a device or a page-locked one: the host maps the
-    pages of the pageable one alone."""
+    """A pageable output beside a device or a page-locked one: the host handles
+    the pages of the pageable one alone."""
     P, lat = _lattice()
     ref = lat.macro()
     outs = [None if k is None else _output(k, lat.ny, lat.nx) for k in kinds]
@@ -94,3 +96,26 @@ def test_initial_temperature_on_any_byte(kind):
     L.lbm_destroy(h)
     lat.close()
     del keep
+
+
+@pytest.mark.parametrize("nx,H", [(61, 30), (301, 398)])
+def test_pageable_outputs_are_written_in_stream_order(nx, H):
+    """Work queued before the read still finds what the outputs held, of a few
+    pages or of many."""
+    import torch
+    P, lat = _lattice(nx=nx, H=H)
+    ref = lat.macro()
+    outs = [_output("pageable", lat.ny, lat.nx) for _ in range(4)]
+    ptr = [C.cast(o[1], C.POINTER(C.c_double)) for o in outs]
+    status = []
+    torch.cuda._sleep(int(1e9))  # about half a second on the lattice's stream
+    reader = threading.Thread(target=lambda: status.append(P.load().lbm_read_macro(lat.handle, *ptr)))
+    reader.start()
+    time.sleep(0.1)
+    seen = [o[0].copy() for o in outs]
+    assert reader.is_alive()
+    reader.join()
+    assert status == [0]
+    for s, o, r in zip(seen, outs, ref):
+        assert (s == -1.1).all() and np.array_equal(o[0], r)
+    lat.close()
