@@ -810,7 +810,7 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
     kp.flags = reinterpret_cast<const uint8_t *>(h->mem + h->lay.off_flags);
     kp.walls = reinterpret_cast<const WallDev *>(h->mem + h->lay.off_walls);
     kp.n_walls = p->n_walls;
-    kp.moving = 0;
+    kp.moving = kp.late = 0;
     for (int k = 0; k < p->n_walls; ++k) kp.moving |= p->walls[k].ux != 0.0 || p->walls[k].uy != 0.0;
     Derived d = derive(p);
     kp.s_e = p->s_e;
@@ -1192,6 +1192,14 @@ lbm_status lbm_debug_bounds_limit(lbm_lattice *h, int64_t bytes) {
     h->kp.blk_hi = h->mem + bytes;
     drop_graph(h);  // a captured graph holds the old range
     h->direct_done = false;
+    return LBM_OK;
+}
+
+lbm_status lbm_debug_late_copies(lbm_lattice *h, int32_t on) {
+    if (!h) return fail(nullptr, LBM_EINVAL, "lattice is NULL");
+    if (on != 0 && on != 1) return fail(h, LBM_EINVAL, "on must be 0 or 1");
+    if (h->batch) return fail(h, LBM_EINVAL, "lattice belongs to a batch");
+    h->kp.late = on;
     return LBM_OK;
 }
 

@@ -86,6 +86,7 @@ struct KParams {
     const WallDev *walls;
     int n_walls;
     int moving;                 // some halfway wall moves (a non-zero Ladd term)
+    int late;                   // test of the tile kernel's report of a copy that does not arrive in time
     // rates and constants
     double s_e, s_nu, s_q, s_eps;     // Eq. 20
     double z_a, z_e, z_nu;            // Eq. 29

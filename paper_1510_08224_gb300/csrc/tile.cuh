@@ -434,13 +434,17 @@ __host__ __device__ constexpr int tile_cols(int k) { return (RX - tile_margin(k)
 template <int RY>
 __host__ __device__ constexpr int tile_rows(int k) { return RY - 2 * k; }
 
+// How a launch runs (bits). Early: read what does not change between steps
+// before waiting for the previous launch (a grid whose blocks can become
+// resident before it ends). Late: every thread but the first takes its region's
+// copy as not arrived in time (a test of the report).
+constexpr int kTileEarly = 1, kTileLate = 2;
+
 // k steps of the tile whose first output cell is (ox, oy), ox a multiple of 4.
-// map: the source buffer's tensor map. early: read what does not change
-// between steps before waiting for the previous launch (a grid whose blocks can
-// become resident before it ends).
+// map: the source buffer's tensor map.
 template <typename S, int TQ, bool BGK, int RX, int RY, int T, typename PA>
 __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const RatesC<float> &r, TileWalls walls,
-                                           const CUtensorMap *map, int k, int ox, int oy, bool early, int *status) {
+                                           const CUtensorMap *map, int k, int ox, int oy, int mode, int *status) {
     using Lay = TileLayout<TQ, RX, RY>;
     extern __shared__ __align__(128) float tile_smem[];
     uint64_t *const bar = reinterpret_cast<uint64_t *>(tile_smem);
@@ -460,6 +464,7 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
         mbar_fence_init();
         *gave_up = 0;
     }
+    const bool early = (mode & kTileEarly) != 0;
     bool any = false;
     auto wall_constants = [&]() {
         for (int n = (int)threadIdx.x; n < (walls.n + 1) * kTileWallWords; n += T) {
@@ -496,7 +501,11 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     }
     if (!early) any = tile_maps<TQ, RX, RY, T>(g, maps, gx0, gy0);
     const bool walled = __syncthreads_or(any);  // also: the barrier is initialised
-    if (boxed && !mbar_wait_bounded(bar, 0)) *gave_up = 1;
+    // a copy that did not arrive in time makes what is stored below invalid: reported by whichever thread saw it
+    if (boxed && (((mode & kTileLate) && threadIdx.x != 0) || !mbar_wait_bounded(bar, 0))) {
+        *gave_up = 1;
+        atomicExch(status, kStatusTimeout);
+    }
     if (HALF && boxed) {
         tile_expand<TQ, RX, RY, T>(pop, gx0 - bx0);
         __syncthreads();
@@ -519,21 +528,18 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     const int x0 = ox - gx0, x1 = min(x0 + tile_cols<RX>(k), g.nx - gx0);
     if (walled) tile_passes<true, S, TQ, BGK, RX, RY, T>(pl, g, r, pop, maps, W, k, gx0, gy0, x0, x1);
     else tile_passes<false, S, TQ, BGK, RX, RY, T>(pl, g, r, pop, maps, W, k, gx0, gy0, x0, x1);
-    // a copy that did not arrive in time (what was stored above is then invalid): report it, with one
-    // more bounded wait so that it cannot land in a later block's shared memory
-    if (*gave_up) {
-        mbar_wait_bounded(bar, 0);
-        if (threadIdx.x == 0) atomicExch(status, kStatusTimeout);
-    }
+    // one more bounded wait for a late copy (a thread that gave up reads its own flag), so that it cannot land
+    // in a later block's shared memory
+    if (*gave_up) mbar_wait_bounded(bar, 0);
 }
 
 template <typename S, int TQ, bool BGK, int RX, int RY, int T, int MINB>
 __global__ void __launch_bounds__(T, MINB)
     k_tile(const Planes<S> pl, const Geom g, const RatesC<float> r, const __grid_constant__ CUtensorMap map,
-           TileWalls walls, int k, int row0, int early, int *status) {
+           TileWalls walls, int k, int row0, int mode, int *status) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     tile_steps<S, TQ, BGK, RX, RY, T>(pl, g, r, walls, &map, k, (int)blockIdx.x * tile_cols<RX>(k),
-                                      row0 + (int)blockIdx.y * tile_rows<RY>(k), early != 0, status);
+                                      row0 + (int)blockIdx.y * tile_rows<RY>(k), mode, status);
 }
 
 }  // namespace nomrt

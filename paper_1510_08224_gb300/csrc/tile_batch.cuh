@@ -57,7 +57,7 @@ struct TileGroup {
     RatesC<float> rc;   // rates shared by the group
     int nlats;
     int k;              // steps of this launch
-    int early;
+    int mode;           // kTileEarly or 0
     int first[kGroupLats + 1];  // first tile of each member; first[nlats]: tiles of the launch
     int *status;
     TileMember lat[kGroupLats];
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(T, MINB) k_tile_batch(const __grid_constant__ 
     RatesC<float> r = P.rc;  // shared rates: parameter-bank operands
     apply_member(r, L.v);
     tile_steps<S, 5, false, RX, RY, T>(pl, g, r, L.walls, &L.map, P.k, bx * tile_cols<RX>(P.k),
-                                       L.row0 + by * tile_rows<RY>(P.k), P.early != 0, P.status);
+                                       L.row0 + by * tile_rows<RY>(P.k), P.mode, P.status);
 }
 
 // The several-steps-per-launch kernels of a batch (MRT, D2Q5).
@@ -140,7 +140,7 @@ struct TileBatchSet<S, ShapeOf<RX, RY, T, MINB>...> {
         G.first[G.nlats] = (int)at;
         if (at == 0) return cudaSuccess;
         G.k = k;
-        G.early = at <= (long long)sms * s.per_sm;
+        G.mode = at <= (long long)sms * s.per_sm ? kTileEarly : 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)at);
         cfg.blockDim = dim3(s.threads);

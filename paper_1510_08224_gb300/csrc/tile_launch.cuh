@@ -222,8 +222,8 @@ cudaError_t launch_tile(TileKernel<S> kern, const TileShape &s, std::atomic<bool
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, make_planes<S>(p, src), make_geom(p), make_rates<float>(p), map,
-                              TileWalls{p.n_walls, p.moving}, k, c.row0, (int)(tiles <= (long long)sms * s.per_sm),
-                              p.status);
+                              TileWalls{p.n_walls, p.moving}, k, c.row0,
+                              (tiles <= (long long)sms * s.per_sm ? kTileEarly : 0) | (p.late ? kTileLate : 0), p.status);
 }
 
 // The shapes of one storage, temperature lattice and collision: region columns

@@ -27,7 +27,7 @@ EXPORTED = ("lbm_footprint_bytes", "lbm_validate", "lbm_create", "lbm_step", "lb
             "lbm_nusselt",
             "lbm_residual", "lbm_get_populations", "lbm_set_populations", "lbm_info", "lbm_steps_per_launch", "lbm_last_error",
             "lbm_destroy", "lbm_residual_fields_noalloc", "lbm_probe_fp64_rate", "lbm_bounds_checking",
-            "lbm_debug_bounds_limit", "lbm_batch_create", "lbm_batch_add", "lbm_batch_remove",
+            "lbm_debug_bounds_limit", "lbm_debug_late_copies", "lbm_batch_create", "lbm_batch_add", "lbm_batch_remove",
             "lbm_batch_set_mode", "lbm_batch_set_kind", "lbm_batch_set_config", "lbm_batch_tune", "lbm_batch_step", "lbm_batch_sync",
             "lbm_batch_info", "lbm_batch_get_mode", "lbm_batch_residuals", "lbm_batch_steps_per_launch",
             "lbm_batch_last_error", "lbm_batch_destroy",
@@ -147,6 +147,8 @@ def load():
         L.lbm_bounds_checking.argtypes = []
         L.lbm_debug_bounds_limit.restype = C.c_int
         L.lbm_debug_bounds_limit.argtypes = [vp, C.c_int64]
+        L.lbm_debug_late_copies.restype = C.c_int
+        L.lbm_debug_late_copies.argtypes = [vp, C.c_int32]
         L.lbm_probe_fp64_rate.restype = C.c_int
         L.lbm_probe_fp64_rate.argtypes = [vp, dp]
         L.lbm_residual_fields_noalloc.restype = C.c_int
@@ -372,6 +374,11 @@ class Lattice:
         n = C.c_int32()
         _check(load().lbm_steps_per_launch(self._h, C.byref(n)), self._h)
         return n.value
+
+    def debug_late_copies(self, on: bool):
+        """Test hook for the timeout path of launches of several steps
+        (lbm_debug_late_copies)."""
+        _check(load().lbm_debug_late_copies(self._h, int(on)), self._h)
 
 
 class Batch:
