@@ -431,7 +431,9 @@ lbm_status lbm_batch_steps_per_launch(lbm_batch *b, int32_t *steps);
 
 /* Wait for the batch's stream; LBM_ETIMEOUT if a persistent launch gave up a
  * grid barrier (the members' state is then undefined; later persistent
- * launches return at once until this call clears the status). */
+ * launches return at once until this call clears the status) or a launch of
+ * several steps the copy of a region (the state of that region's member is then
+ * undefined, and the member's own read-outs report it too until this call has). */
 lbm_status lbm_batch_sync(lbm_batch *b);
 
 /* Test hook for the timeout path. With extra = 1 the persistent kernel's grid

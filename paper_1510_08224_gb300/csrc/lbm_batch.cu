@@ -581,6 +581,8 @@ void plan_tiles(lbm_batch *b) {
                 t.plane = h->kp.plane;
                 t.v = G.lat[m].v;
                 t.walls = nomrt::TileWalls{h->kp.n_walls, h->kp.moving};
+                t.status = h->kp.status;
+                t.late = h->kp.late ? nomrt::kTileLate : 0;
                 t.row0 = h->kp.py ? 0 : 1;
             }
         }
@@ -1011,6 +1013,9 @@ lbm_status lbm_batch_sync(lbm_batch *b) {
         const int zero = 0;
         cudaMemcpy(b->d_status, &zero, sizeof zero, cudaMemcpyHostToDevice);
         cudaMemset(b->d_bar, 0, 4 * sizeof(unsigned));
+        // what the members' own words hold is reported with it
+        for (lbm_lattice *h : b->members)
+            cudaMemcpy(h->kp.status, &zero, sizeof zero, cudaMemcpyHostToDevice);
         return bfail(b, LBM_ETIMEOUT, "a batch kernel gave up a bounded wait (a grid barrier or a copy)");
     }
     if constexpr (nomrt::kBoundsBuild) {

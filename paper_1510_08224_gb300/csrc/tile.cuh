@@ -441,10 +441,12 @@ __host__ __device__ constexpr int tile_rows(int k) { return RY - 2 * k; }
 constexpr int kTileEarly = 1, kTileLate = 2;
 
 // k steps of the tile whose first output cell is (ox, oy), ox a multiple of 4.
-// map: the source buffer's tensor map.
+// map: the source buffer's tensor map. status: the word a late copy is reported
+// to; also: another, or NULL (a batch's beside its member's).
 template <typename S, int TQ, bool BGK, int RX, int RY, int T, typename PA>
 __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const RatesC<float> &r, TileWalls walls,
-                                           const CUtensorMap *map, int k, int ox, int oy, int mode, int *status) {
+                                           const CUtensorMap *map, int k, int ox, int oy, int mode, int *status,
+                                           int *also = nullptr) {
     using Lay = TileLayout<TQ, RX, RY>;
     extern __shared__ __align__(128) float tile_smem[];
     uint64_t *const bar = reinterpret_cast<uint64_t *>(tile_smem);
@@ -505,6 +507,7 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     if (boxed && (((mode & kTileLate) && threadIdx.x != 0) || !mbar_wait_bounded(bar, 0))) {
         *gave_up = 1;
         atomicExch(status, kStatusTimeout);
+        if (also) atomicExch(also, kStatusTimeout);
     }
     if (HALF && boxed) {
         tile_expand<TQ, RX, RY, T>(pop, gx0 - bx0);

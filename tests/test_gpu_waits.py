@@ -1,7 +1,7 @@
 """A region's copy that does not arrive in time (launches of several steps): the
 test hook makes the bounded wait of every thread but one give up at once; the
 kernel returns normally, the next synchronising call reports LBM_ETIMEOUT once,
-and the lattice works again."""
+and the lattice works again. In a batch both the batch and the member report."""
 import numpy as np
 import pytest
 
@@ -50,3 +50,42 @@ def test_late_copy_is_reported_by_any_thread(name, storage, steps):
     side.synchronize()
     for u, v in zip(a.populations(), b.populations()):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("first", ["member", "batch"])
+def test_late_copy_of_a_member_is_reported_by_member_and_batch(first, storage):
+    import paper_1510_08224_gb300 as P
+    cases = [_case("cavity"), _case("box"), lc.cavity(n=40, Ra=1e4, noise=1e-3)]
+    lats = [P.Lattice(c, storage=storage) for c in cases]
+    lats[1].debug_late_copies(True)
+    b = P.Batch()
+    for lat in lats:
+        b.add(lat)
+    with pytest.raises(P.LBMError):  # a member's hook is set before it joins
+        lats[1].debug_late_copies(False)
+    b.step(8)
+    lats[0].macro(), lats[2].residual()
+    if first == "member":
+        for read in (lats[1].macro, b.sync):
+            _timed_out(P, read)
+    else:
+        _timed_out(P, b.residuals)
+    b.sync()
+    for lat in lats:  # reported once
+        lat.macro()
+    b.remove(lats[1])
+    lats[1].debug_late_copies(False)
+    b.add(lats[1])
+    states = [lc.random_state(c, seed=20 + i) for i, c in enumerate(cases)]
+    for lat, s in zip(lats, states):
+        lat.set_populations(*s)
+    b.step(8)
+    b.sync()
+    for lat, c, s in zip(lats, cases, states):
+        ref = P.Lattice(c, storage=storage)
+        ref.set_populations(*s)
+        ref.step(8)
+        for u, v in zip(lat.populations(), ref.populations()):
+            assert np.array_equal(u, v)
+    b.close()
