@@ -449,8 +449,6 @@ def run_batched(args):
               flush=True)
         return 0
     tuned_kind, tuned_cfg, ms_cand = b.tune(trial_steps=64)
-    if tuned_kind == "fused" and b.steps_per_launch() > 1:
-        tuned_cfg = -1  # several steps per launch
     tuned_unit = b.info()["rows_per_unit"]
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)

@@ -416,9 +416,11 @@ lbm_status lbm_batch_get_member_kernel(const lbm_batch *b, int32_t *variant, int
  * one-segment units, PERSISTENT 0-4 with two-segment units, CONCURRENT own,
  * CONCURRENT VEC4 0-4, CONCURRENT VEC4W 0-4; +inf for a
  * candidate that cannot run, such as PERSISTENT with node-based walls). The
- * FUSED kind's several steps per launch are timed too and, where fastest, kept
- * (config -1; *best_config then holds the config of its single steps). Any
- * output may be NULL. Synchronises. */
+ * FUSED kind's several steps per launch are timed too and, where fastest, kept:
+ * *best_config is then -1, the default config. lbm_batch_set_kind and
+ * lbm_batch_set_config with what is returned change nothing (CONCURRENT aside,
+ * whose *best_config names a member kernel). Any output may be NULL.
+ * Synchronises. */
 lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *best_kind, int32_t *best_config,
                           float *ms_per_step);
 

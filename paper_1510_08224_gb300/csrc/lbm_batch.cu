@@ -1167,7 +1167,7 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, int32_t *best_kind,
     }
     drop_graph(b);
     if (best_kind) *best_kind = b->kind;
-    if (best_config) *best_config = b->kind == LBM_BATCH_CONCURRENT ? best - kConc - 1 : b->cfg();
+    if (best_config) *best_config = b->kind == LBM_BATCH_CONCURRENT ? best - kConc - 1 : b->config;
     if (ms_per_step)
         for (int c = 0; c < kCand; ++c) ms_per_step[c] = ms[c];
     return LBM_OK;

@@ -464,7 +464,8 @@ class Batch:
         concurrent_vec4_cfg0-4 and concurrent_vec4w_cfg0-4; for the concurrent
         kind the config is -1 (own), 0-4 (vec4) or 5-9 (vec4w), already in
         force as the member kernel. The fused kind's several steps per launch
-        are timed too and, where fastest, kept (steps_per_launch() then says so)."""
+        are timed too and, where fastest, kept: the config is then -1, the
+        default."""
         kind, cfg = C.c_int32(), C.c_int32()
         ms = (C.c_float * 31)()
         self._check(load().lbm_batch_tune(self._h, int(trial_steps), C.byref(kind), C.byref(cfg), ms))
