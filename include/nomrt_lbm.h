@@ -163,9 +163,11 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
 /* Advance nsteps >= 0 time steps (Eqs. 8-9 and 24-25, fused). Asynchronous on the
  * lattice's stream. With the AUTO step kernel, runs of two steps or more of an
  * FP32 or FP16 lattice without node-based walls (and with at most 15 walls; in
- * FP16 up to 6.5 million cells, 4 million with nine temperature populations) take up to eight steps per launch, tile by tile in
- * shared memory, the tile and the steps per launch chosen from the lattice's
- * size; the bits are those of single steps. Every other step is one kernel,
+ * FP16 up to 6.5 million cells, 4 million with nine temperature populations) take
+ * up to eight steps per launch, tile by tile in shared memory, the tile and the
+ * steps per launch chosen from the lattice's size, unless that says that single
+ * steps are faster (wide lattices of few rows); the bits are those of single
+ * steps. Every other step is one kernel,
  * plus one for the boundary nodes of node-based walls; runs of 4 such steps or
  * more replay CUDA graphs of 32 and of 4 steps, captured once per step-kernel
  * choice (the same kernels and bits, without the launch gap between steps; a
@@ -352,8 +354,8 @@ lbm_status lbm_batch_remove(lbm_batch *b, lbm_lattice *h);
 /* How a batch step runs.
  * FUSED (the default): one kernel launch per launch group for up to eight
  * steps, each block updating one tile of a member in shared memory; where a
- * member has node-based walls or more than 15 walls, or a config is set, one
- * launch per step, one 128-thread block of the four-cell row code per 512-cell
+ * member has node-based walls or more than 15 walls, the members' sizes favour
+ * single steps, or a config is set, one launch per step, one 128-thread block of the four-cell row code per 512-cell
  * row segment of every member (a 1-D grid over the members' segments). The bits
  * are the same.
  * PERSISTENT: one cooperative launch per group for steps_per_launch steps: its

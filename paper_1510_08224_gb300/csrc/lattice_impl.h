@@ -61,7 +61,7 @@ struct lbm_lattice {
     // several steps per launch (AUTO): the plan for this lattice (shape -1: none), made at the first
     // run of two steps or more, and the tensor maps of its two buffers
     const nomrt::TileLaunchers *tile = nullptr;
-    nomrt::TilePlan tile_plan{-1, 0};
+    nomrt::TilePlan tile_plan;
     bool tile_planned = false;
     CUtensorMap tile_map[2];
     bool recorded = false;  // some run was recorded into a caller's graph

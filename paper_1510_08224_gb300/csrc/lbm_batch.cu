@@ -489,7 +489,7 @@ struct lbm_batch {
     std::vector<nomrt::GroupParams> groups;  // launch parameters, kGroupLats members each
     // FUSED, default config: several steps per launch where every member can (shape -1: not). One launch
     // descriptor per group and batch-step parity, tiles[2 g + parity]
-    nomrt::TilePlan tile_plan{-1, 0};
+    nomrt::TilePlan tile_plan;
     std::vector<nomrt::TileGroup> tiles;
     std::vector<size_t> member_of;  // member index of slot m of group g, at g kGroupLats + m
     int64_t cells = 0;
@@ -541,7 +541,7 @@ void drop_graph(lbm_batch *b) {
 
 // The several-steps-per-launch plan and descriptors of the launch groups.
 void plan_tiles(lbm_batch *b) {
-    b->tile_plan = nomrt::TilePlan{-1, 0};
+    b->tile_plan = nomrt::TilePlan{};
     b->tiles.clear();
     const nomrt::TileBatchLaunchers *L = nomrt::tile_batch_launchers(b->storage);
     std::vector<const nomrt::KParams *> kp;

@@ -110,7 +110,7 @@ struct KParams {
 // How a lattice steps several times per launch: a tile shape (an index, -1: it
 // does not) and the steps per launch.
 struct TilePlan {
-    int shape, steps;
+    int shape = -1, steps = 0;
 };
 
 // The several-steps-per-launch kernels (tile.cuh) of one storage, temperature

@@ -68,6 +68,44 @@ inline double tile_cycles(const TileShape &s, int k, long long tiles, int nq, do
            0.5 * wave(s.per_sm);
 }
 
+// Estimated cycles of a single step of the lattices in one launch, as graphs
+// replay it: the populations of the rows with cells, read and written, and
+// those of wall rows, written, at HBM's rate (FP16 in whole blocks of 512 cells,
+// whose conversions take as long in a block that is not full); at least a
+// block's own cost per row of 512 cells; and a launch's latency.
+inline double single_cycles(const KParams *const *lats, int n, int nq, int elem, int sms) {
+    constexpr double kHbm = 21.2, kRowBlock = 315;  // bytes and cycles per SM
+    const double launch = elem == 4 ? 5200 : 6200, least = elem == 4 ? 11400 : 9900;
+    double bytes = 0, blocks = 0;
+    for (int m = 0; m < n; ++m) {
+        const KParams &p = *lats[m];
+        const int rows = tile_cover(p).rows, segments = (p.pitch + 511) / 512;
+        if (rows <= 0) continue;
+        bytes += 2.0 * nq * elem * (elem == 4 ? p.nx : 512.0 * segments) * (rows + 0.5 * (p.ny - rows));
+        blocks += (double)p.ny * segments;
+    }
+    return std::max(least, launch + std::max(bytes / (kHbm * sms), blocks * kRowBlock / sms));
+}
+
+// The share of a single step's estimate that a step of the tiles may take. A
+// tile does the work of all its rows whatever the lattice has, so wide lattices
+// of few rows are faster stepped singly; the line lies where 150 timed pairs
+// cross (145 on the faster side, the worst at 1.25 times the other), and no
+// lattice of 0.15 to 7 times as many columns as rows comes near it. FP16 tiles
+// take their estimate's 1.2 to 1.7 times in one or two rows of tiles. Measured,
+// us a step, tiles / single steps (and the estimates' ratio): FP32 262144 columns
+// x 14 rows 46 / 67 (0.50), x 6 39 / 33 (0.99), x 4 38 / 22 (1.34), 1048576 x 4 146 / 91
+// (1.38), 4194304 x 2 570 / 211 (2.30), 20000 x 4 4.1 / 6.1 (0.70), nine temperature
+// populations 60000 x 10 16.6 / 16.3 (0.73), x 8 15.0 / 12.0 (0.81); FP16 65536 x 32
+// 24.5 / 26.1 (0.87), 60000 x 20 19.4 / 12.7 (0.95), x 4 11.7 / 5.9 (1.58), 262144 x 4 45 /
+// 14 (2.35), but nine populations 485 x 870 7.9 / 9.5 (0.98).
+inline double tile_share(const KParams *const *lats, int n, int elem) {
+    if (elem == 4) return 0.76;
+    for (int m = 0; m < n; ++m)
+        if (tile_cover(*lats[m]).rows > 32) return 1.0;
+    return 0.89;
+}
+
 constexpr int kTileMaxSteps = 8;
 constexpr double kL2Bytes = 100e6;  // what of the 129 MB L2 two buffers can count on
 
@@ -81,15 +119,15 @@ constexpr double kL2Bytes = 100e6;  // what of the 129 MB L2 two buffers can cou
 // 300^2: 120 -> 76) and have no such limit.
 inline double tile_most_f16(int nq) { return nq <= 14 ? 6.5e6 : 4.0e6; }
 
-// The shape and steps per launch with the least estimated time per step.
-// Lattices with node-based walls or more walls than a block keeps step once per
+// The shape and steps per launch with the least estimated time per step, or shape
+// -1 where single steps are estimated faster. Lattices with node-based walls or more walls than a block keeps step once per
 // launch. FP16: several regions of 32 rows per SM only where they make more than
 // two waves; below, the estimate misjudges them (600^2: 6.1 us a step against
 // 5.7; 256^2 with nine temperature populations 3.3 against 3.0; but 1111 x 333
 // 7.8 against 8.2).
 inline TilePlan choose_tile(const KParams *const *lats, int n, bool batch, int nq, int elem, const TileShape *shapes,
                             int n_shapes, int sms) {
-    TilePlan best{-1, 0};
+    TilePlan best;
     double least = 0, cells = 0;
     if (n < 1 || sms <= 0) return best;
     for (int m = 0; m < n; ++m) {
@@ -101,28 +139,35 @@ inline TilePlan choose_tile(const KParams *const *lats, int n, bool batch, int n
     if (elem == 2 && !batch && cells > tile_most_f16(nq)) return best;
     const double cell_bytes = 2.0 * nq * elem;
     const bool fits_l2 = cell_bytes * cells < kL2Bytes;
+    // tiles of a launch of k steps (-1: more than a launch can have)
+    auto count = [&](const TileShape &s, int k) -> long long {
+        const int tx = shape_cols(s, k), ty = shape_rows(s, k);
+        long long tiles = 0;
+        for (int m = 0; m < n; ++m) {
+            const TileCover c = tile_cover(*lats[m]);
+            if (c.rows <= 0 || c.cols <= 0) continue;
+            const long long gx = (c.cols + tx - 1) / tx, gy = (c.rows + ty - 1) / ty;
+            if (!batch && gy > 65535) return -1;  // a lattice alone: the launch grid's y limit
+            tiles += gx * gy;
+        }
+        return tiles > 0x3FFFFFFF ? -1 : tiles;
+    };
     for (int i = 0; i < n_shapes; ++i)
         for (int k = 2; k <= kTileMaxSteps; ++k) {
-            const int tx = shape_cols(shapes[i], k), ty = shape_rows(shapes[i], k);
-            if (tx < 4 || ty < 2) break;
-            long long tiles = 0;
-            bool fits = true;
-            for (int m = 0; m < n; ++m) {
-                const TileCover c = tile_cover(*lats[m]);
-                if (c.rows <= 0 || c.cols <= 0) continue;
-                const long long gx = (c.cols + tx - 1) / tx, gy = (c.rows + ty - 1) / ty;
-                fits = fits && (batch || gy <= 65535);  // a lattice alone: the launch grid's y limit
-                tiles += gx * gy;
-            }
-            if (!fits || tiles > 0x3FFFFFFF) continue;
+            if (shape_cols(shapes[i], k) < 4 || shape_rows(shapes[i], k) < 2) break;
+            const long long tiles = count(shapes[i], k);
+            if (tiles < 0) continue;
             if (elem == 2 && shapes[i].ry >= 32 && shapes[i].per_sm > 1 && tiles <= 2LL * sms * shapes[i].per_sm)
                 continue;
             const double t = tile_cycles(shapes[i], k, tiles, nq, cell_bytes, fits_l2, sms) / k;
             if (best.shape < 0 || t < least) {
-                best = TilePlan{i, k};
+                best.shape = i;
+                best.steps = k;
                 least = t;
             }
         }
+    if (best.shape < 0) return best;
+    if (least > tile_share(lats, n, elem) * single_cycles(lats, n, nq, elem, sms)) return TilePlan{};
     return best;
 }
 
