@@ -559,12 +559,14 @@ bool plan_tiles(lbm_lattice *h) {
 // n >= 2 steps as evenly sized launches of at most tile_plan.steps steps. Once a
 // run has been recorded into a caller's graph, as many launches as steps modulo
 // 2: an even run then ends on the buffer it began on, so that the graph of one
-// can be replayed with other even runs between. Each is a programmatic dependent
-// of the one before and costs the GPU more time than its launch costs the host,
-// so they are launched directly.
+// can be replayed with other even runs between (where that makes it launches of
+// one step, single steps unless the plan says that they are slower). Each is a
+// programmatic dependent of the one before and costs the GPU more time than its
+// launch costs the host, so they are launched directly.
 lbm_status step_tiles(lbm_lattice *h, int64_t n) {
     int64_t launches = (n + h->tile_plan.steps - 1) / h->tile_plan.steps;
     if (h->recorded) launches += (launches ^ n) & 1;
+    if (launches == n && !h->tile_plan.one) return step_direct(h, n);
     for (int64_t i = launches; i > 0; --i) {
         const int k = (int)((n + i - 1) / i);
         cudaError_t e = h->tile->launch(h->kp, h->tile_plan.shape, h->tile_map[h->cur], h->cur, k, h->stream);

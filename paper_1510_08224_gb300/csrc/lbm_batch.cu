@@ -787,10 +787,12 @@ cudaError_t launch_tile_steps(lbm_batch *b, int parity, int k, cudaStream_t st) 
 
 cudaError_t launch_steps(lbm_batch *b, int parity, int n, cudaStream_t st) {
     if (b->kind == LBM_BATCH_CONCURRENT) return launch_concurrent(b, n, st, true);
-    if (b->kind == LBM_BATCH_FUSED && b->config < 0 && b->tile_plan.shape >= 0 && n > 1) {
-        // as many launches as steps modulo 2, so that the buffers' parity stays that of the steps
-        int launches = (n + b->tile_plan.steps - 1) / b->tile_plan.steps;
-        launches += (launches ^ n) & 1;
+    // several steps per launch: as many launches as steps modulo 2, so that the buffers' parity stays that of
+    // the steps (where that makes it launches of one step, single steps unless the plan says that they are slower)
+    int launches = b->tile_plan.shape >= 0 ? (n + b->tile_plan.steps - 1) / b->tile_plan.steps : n;
+    launches += (launches ^ n) & 1;
+    if (b->kind == LBM_BATCH_FUSED && b->config < 0 && b->tile_plan.shape >= 0 && n > 1 &&
+        (launches < n || b->tile_plan.one)) {
         for (int i = launches; i > 0; --i) {
             const int k = (n + i - 1) / i;
             cudaError_t e = launch_tile_steps(b, parity, k, st);

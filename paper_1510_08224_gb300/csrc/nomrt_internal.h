@@ -108,9 +108,11 @@ struct KParams {
 };
 
 // How a lattice steps several times per launch: a tile shape (an index, -1: it
-// does not) and the steps per launch.
+// does not) and the steps per launch, and whether launches of one step each are
+// faster than single steps.
 struct TilePlan {
     int shape = -1, steps = 0;
+    bool one = false;
 };
 
 // The several-steps-per-launch kernels (tile.cuh) of one storage, temperature

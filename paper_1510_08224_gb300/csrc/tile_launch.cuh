@@ -167,7 +167,16 @@ inline TilePlan choose_tile(const KParams *const *lats, int n, bool batch, int n
             }
         }
     if (best.shape < 0) return best;
-    if (least > tile_share(lats, n, elem) * single_cycles(lats, n, nq, elem, sms)) return TilePlan{};
+    const double single = single_cycles(lats, n, nq, elem, sms);
+    if (least > tile_share(lats, n, elem) * single) return TilePlan{};
+    // launches of one step (two steps that have to end on the buffer they began on): by the same estimates, or
+    // up to one wave of tiles, FP16 two, where single steps launched one by one take longer than replayed (24
+    // lattices of 32 to 128: 7.7 us a step against 10.2; 8 of 200 to 400, 1.8 waves, FP32 14.8 / 14.4, FP16 14.9
+    // / 15.9; 64 of 128 to 1024 FP16 393 / 352; one of 4 x 262144 172 / 250)
+    const TileShape &s = shapes[best.shape];
+    const long long tiles = count(s, 1);
+    best.one = tiles >= 0 && (tiles <= (elem == 2 ? 2LL : 1LL) * sms * s.per_sm ||
+                              tile_cycles(s, 1, tiles, nq, cell_bytes, fits_l2, sms) <= 0.76 * single);
     return best;
 }
 

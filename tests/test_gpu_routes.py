@@ -50,3 +50,34 @@ def test_wide_lattices_of_few_rows_take_single_steps(model, storage):
         b.remove(lats[0])
         assert b.steps_per_launch() > 1
         b.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("side", [60, 700])
+def test_two_steps_that_end_on_their_first_buffer(side, storage):
+    """A batch's run of two steps, and a lattice's once a run was recorded: two
+    launches of one step on small lattices, single steps on large ones."""
+    import torch
+    import paper_1510_08224_gb300 as P
+    case = lc.cavity(n=side, n_y=side - 9, Ra=1e4, noise=1e-3)
+    f0, g0 = lc.random_state(case, seed=9)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        a, b, c = (P.Lattice(case, storage=storage, stream=stream) for _ in range(3))
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            a.step(2)
+        batch = P.Batch(stream=stream)
+        c.set_step_kernel("scalar")
+        for lat in (a, b, c):
+            lat.set_populations(f0, g0)
+        batch.add(b)
+        for n in (2, 2, 3, 1, 2):  # ends on the buffer the recorded run began on
+            a.step(n), batch.step(n), c.step(n)
+        graph.replay(), c.step(2), batch.step(2)
+    stream.synchronize()
+    want = c.populations()
+    for lat in (a, b):
+        for u, v in zip(lat.populations(), want):
+            assert np.array_equal(u, v)
+    batch.close()
