@@ -237,7 +237,8 @@ cudaError_t launch_dependent(K kern, dim3 grid, cudaStream_t st, A... args) {
 
 template <typename S, int MINB, int TQ, bool BGK>
 cudaError_t launch_step4(dim3 grid, cudaStream_t st, const Planes<S> &pl, const Geom &g, const RatesC<float> &r) {
-    return launch_dependent<MINB>(k_step4<S, MINB, TQ, BGK>, grid, st, pl, g, r);
+    using Own = typename StepRates<S, TQ, BGK, MINB <= (sizeof(S) == 2 ? 4 : 5)>::type;
+    return launch_dependent<MINB>(k_step4<S, MINB, TQ, BGK>, grid, st, pl, g, Own(r));
 }
 
 // The per-warp form: one 128-cell row segment per warp, four per block.
@@ -247,8 +248,9 @@ cudaError_t launch_step4w(const KParams &p, int src, cudaStream_t st) {
     const long long nunits = (long long)p.ny * upr;
     if (nunits > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)((nunits + 3) / 4));
+    using Own = typename StepRates<S, TQ, BGK, sizeof(S) == 4 && MINB <= 7>::type;
     return launch_dependent<MINB>(k_step4w<S, MINB, TQ, BGK>, grid, st, make_planes<S>(p, src), make_geom(p),
-                                  make_rates<float>(p), upr, (int)nunits);
+                                  Own(make_rates<float>(p)), upr, (int)nunits);
 }
 
 // TQ: temperature populations per node (5: D2Q5; 9: the D2Q9 model). BGK:
@@ -306,7 +308,8 @@ cudaError_t launch_step_m(const KParams &p, int variant, int src, cudaStream_t s
     const int gy = (p.ny + (int)b.y - 1) / (int)b.y;
     const dim3 grid((p.nx + b.x - 1) / b.x, gy < 65535 ? gy : 65535);
     if (variant != kStepScalar && variant != kStepAuto) return cudaErrorInvalidValue;
-    k_step<S, TQ, BGK><<<grid, b, 0, st>>>(make_planes<S>(p, src), make_geom(p), make_rates<C>(p));
+    using Own = typename StepRates<S, TQ, BGK, TQ == 9 && BGK>::type;
+    k_step<S, TQ, BGK><<<grid, b, 0, st>>>(make_planes<S>(p, src), make_geom(p), Own(make_rates<C>(p)));
     return cudaGetLastError();
 }
 

@@ -18,6 +18,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "nomrt_internal.h"
 
 namespace nomrt {
@@ -164,6 +166,69 @@ inline RatesC<C> make_rates(const KParams &p) {
     r.theta = (C)p.theta;
     return r;
 }
+
+// The rates of single-step kernels that keep their own, of at most 128 bytes: a
+// larger parameter of this kind changes how the compiler schedules the loads of
+// the whole kernel. Measured with RatesC against these, us a step: FP32 VEC4W
+// 1402^2 38.7 -> 37.5, VEC4 4194304 x 4 228 -> 211; FP16 with nine temperature
+// populations 4096 x 2048 98.8 -> 93.2, 2048 x 1024 32.5 -> 30.3 (BGK 94.1 -> 93.0,
+// 30.9 -> 30.0; one cell per thread 218 -> 184). The kernels not listed at StepRates
+// lose by the change or spill either way.
+
+// FP32, MRT, D2Q5.
+struct RatesMrt {
+    float hx, hFy0, hg_beta, T_ref, om_a, z_a;
+    float om_e4, om_nu4, om_q4, om_eps4, s_e4, s_nu4, ns_nu4, s_q2, s_eps4;
+    float h_e, h_nu2, nh_nu, h3eps, om_ze4, zv_e4, om_zn4;
+    explicit RatesMrt(const RatesC<float> &r)
+        : hx(r.hx), hFy0(r.hFy0), hg_beta(r.hg_beta), T_ref(r.T_ref), om_a(r.om_a), z_a(r.z_a), om_e4(r.om_e4),
+          om_nu4(r.om_nu4), om_q4(r.om_q4), om_eps4(r.om_eps4), s_e4(r.s_e4), s_nu4(r.s_nu4), ns_nu4(r.ns_nu4),
+          s_q2(r.s_q2), s_eps4(r.s_eps4), h_e(r.h_e), h_nu2(r.h_nu2), nh_nu(r.nh_nu), h3eps(r.h3eps),
+          om_ze4(r.om_ze4), zv_e4(r.zv_e4), om_zn4(r.om_zn4) {}
+};
+
+// FP16 with nine temperature populations, MRT: the rates unfolded (collide_u).
+struct RatesHalf9 {
+    float om_e, om_nu, om_q, om_eps, s_e, s_nu, s_q, s_eps;  // 1 - s_k, s_k
+    float h_nu, om_a, z_a, om_ze, om_zn;
+    float ax, Fy0, g_beta, T_ref, hx;
+    float h2e, h2nu, h23eps;  // 2 (1 - s_e/2), 2 (1 - s_nu/2), (2/3)(1 - s_eps/2)
+    float z_e, z_nu, om_zq, z_q, om_zeps, z_eps, theta;
+    explicit RatesHalf9(const RatesC<float> &r)
+        : om_e(4 * r.om_e4), om_nu(r.om_nu), om_q(4 * r.om_q4), om_eps(4 * r.om_eps4), s_e(4 * r.s_e4), s_nu(r.s_nu),
+          s_q(2 * r.s_q2), s_eps(4 * r.s_eps4), h_nu(r.h_nu), om_a(r.om_a), z_a(r.z_a), om_ze(r.om_ze),
+          om_zn(r.om_zn), ax(r.ax), Fy0(r.Fy0), g_beta(r.g_beta), T_ref(r.T_ref), hx(r.hx), h2e(2 * r.h_e),
+          h2nu(2 * r.h_nu), h23eps(2 * r.h3eps), z_e(r.z_e), z_nu(r.z_nu), om_zq(r.om_zq), z_q(r.z_q),
+          om_zeps(r.om_zeps), z_eps(r.z_eps), theta(r.theta) {}
+};
+
+// FP16 with nine temperature populations, BGK.
+struct RatesHalf9Bgk {
+    float om_nu, s_nu, h_nu, om_a, z_a, ax, Fy0, g_beta, T_ref, hx, theta;
+    explicit RatesHalf9Bgk(const RatesC<float> &r)
+        : om_nu(r.om_nu), s_nu(r.s_nu), h_nu(r.h_nu), om_a(r.om_a), z_a(r.z_a), ax(r.ax), Fy0(r.Fy0),
+          g_beta(r.g_beta), T_ref(r.T_ref), hx(r.hx), theta(r.theta) {}
+};
+static_assert(sizeof(RatesMrt) <= 128 && sizeof(RatesHalf9) <= 128, "rates of a kernel's own");
+
+// The rates a single-step kernel takes (OWN: one of those named above, as the
+// kernel says).
+template <typename S, int TQ, bool BGK, bool OWN>
+struct StepRates {
+    using type = RatesC<typename Store<S>::C>;
+};
+template <>
+struct StepRates<float, 5, false, true> {
+    using type = RatesMrt;
+};
+template <>
+struct StepRates<__half, 9, false, true> {
+    using type = RatesHalf9;
+};
+template <>
+struct StepRates<__half, 9, true, true> {
+    using type = RatesHalf9Bgk;
+};
 
 // Kernel arguments: typed plane pointers of both buffers.
 template <typename S>
@@ -606,6 +671,76 @@ __device__ __forceinline__ void collide_x(const R &r, T f[9], T t[TQ]) {
     }
 }
 
+// collide_x's MRT flow collision with the rates unfolded, for FP16 with nine
+// temperature populations: a power-of-two factor moves through a rounding
+// unchanged, so the bits are the same, 113 operations in place of 101, but the
+// kernel's loads are scheduled better around it (4096 x 2048 95.8 -> 93.2 us a
+// step with rates of the same size, 2048 x 1024 32.0 -> 30.3).
+template <typename T>
+__device__ __forceinline__ void collide_u(const RatesHalf9 &r, T f[9], T t[9]) {
+    using O = Ops<T>;
+    const T n0 = O::add(O::add(O::add(O::add(t[0], t[1]), O::add(t[2], t[3])), O::add(t[4], t[5])),
+                        O::add(O::add(t[6], t[7]), t[8]));  // T - T_ref
+    const T Fx = O::bc(r.ax);
+    const T Fy = O::fma(O::bc(r.g_beta), n0, O::bc(r.Fy0));  // Eq. 4
+    // D2Q9 forward map (Eq. 13)
+    const T a13 = O::add(f[1], f[3]), d13 = O::sub(f[1], f[3]);
+    const T a24 = O::add(f[2], f[4]), d24 = O::sub(f[2], f[4]);
+    const T a57 = O::add(f[5], f[7]), d57 = O::sub(f[5], f[7]);
+    const T a68 = O::add(f[6], f[8]), d68 = O::sub(f[6], f[8]);
+    const T D = O::add(a57, a68);
+    const T A4 = O::add(a13, a24);
+    const T m0 = O::add(O::add(f[0], A4), D);
+    const T m6 = O::add(d57, d68);
+    const T m7 = O::sub(d57, d68);
+    const T jx = O::add(d13, m7);
+    const T jy = O::add(d24, m6);
+    const T m3 = O::add(A4, O::add(D, D));
+    const T m4 = O::sub(a13, a24);
+    const T m5 = O::sub(a57, a68);
+    // Eq. 19 with rho0 = 1
+    const T ux = O::add(jx, O::bc(r.hx));
+    const T uy = O::fma(O::bc(0.5f), Fy, jy);
+    const T uyuy = O::mul(uy, uy);
+    const T uu = O::fma(ux, ux, uyuy);
+    const T uF = O::fma(ux, Fx, O::mul(uy, Fy));
+    // Eq. 8
+    const T p1 = O::add(jx, Fx);
+    const T p2 = O::add(jy, Fy);
+    const T p3 = O::fma(O::bc(r.om_e), m3,
+                        O::fma(O::bc(r.s_e), O::fma(O::bc(2.0f / 3.0f), m0, uu), O::mul(O::bc(r.h2e), uF)));
+    const T dxy = O::fma(ux, ux, O::mul(O::bc(-1.f), uyuy));
+    const T dF = O::fma(ux, Fx, O::mul(O::bc(-1.f), O::mul(uy, Fy)));
+    const T p4 = O::fma(O::bc(r.om_nu), m4, O::fma(O::bc(r.s_nu), dxy, O::mul(O::bc(r.h2nu), dF)));
+    const T cF = O::fma(ux, Fy, O::mul(uy, Fx));
+    const T p5 = O::fma(O::bc(r.om_nu), m5, O::fma(O::bc(r.s_nu), O::mul(ux, uy), O::mul(O::bc(r.h_nu), cF)));
+    const T p6 = O::fma(O::bc(r.om_q), m6, O::mul(O::bc(1.0f / 3.0f), O::fma(O::bc(r.s_q), jy, Fy)));
+    const T p7 = O::fma(O::bc(r.om_q), m7, O::mul(O::bc(1.0f / 3.0f), O::fma(O::bc(r.s_q), jx, Fx)));
+    const T p8 = O::fma(O::bc(r.om_eps), D,
+                        O::fma(O::bc(r.s_eps), O::fma(O::bc(1.0f / 9.0f), m0, O::mul(O::bc(1.0f / 3.0f), uu)),
+                               O::mul(O::bc(r.h23eps), uF)));
+    // back map (Eq. A1); the 1/2 and 1/4 scalings are exact
+    const T A = O::fma(O::bc(0.25f), p3, O::mul(O::bc(-0.5f), p8));
+    const T B = O::mul(O::bc(0.25f), p4);
+    const T h1 = O::mul(O::bc(0.5f), O::sub(p1, p7));
+    const T h2 = O::mul(O::bc(0.5f), O::sub(p2, p6));
+    const T P = O::mul(O::bc(0.25f), O::add(p8, p5));
+    const T Q = O::mul(O::bc(0.25f), O::add(p6, p7));
+    const T Rm = O::mul(O::bc(0.25f), O::sub(p8, p5));
+    const T Sx = O::mul(O::bc(0.25f), O::sub(p6, p7));
+    const T AB = O::add(A, B), AmB = O::sub(A, B);
+    f[0] = O::add(O::sub(m0, p3), p8);
+    f[1] = O::add(AB, h1);
+    f[3] = O::sub(AB, h1);
+    f[2] = O::add(AmB, h2);
+    f[4] = O::sub(AmB, h2);
+    f[5] = O::add(P, Q);
+    f[7] = O::sub(P, Q);
+    f[6] = O::add(Rm, Sx);
+    f[8] = O::sub(Rm, Sx);
+    thermal_q9_x<T>(r, t, n0, ux, uy, uu);
+}
+
 // The MRT collision with the D2Q5 temperature lattice in FP64: collide_x's
 // moments with the products regrouped for the fewest operations, 94 instead of
 // 101 (FP64 steps are bound by that pipe: two lanes per cycle and SM). The terms
@@ -774,24 +909,26 @@ __device__ __forceinline__ void collide_bgk_x(const R &r, T f[9], T t[TQ]) {
 }
 
 // The collision of one cell in the storage's compute type: MRT or BGK.
-template <typename S, int TQ, bool BGK>
-__device__ __forceinline__ void collide_cell(const RatesC<typename Store<S>::C> &r, typename Store<S>::C f[9],
+template <typename S, int TQ, bool BGK, typename R>
+__device__ __forceinline__ void collide_cell(const R &r, typename Store<S>::C f[9],
                                              typename Store<S>::C t[TQ]) {
     using C = typename Store<S>::C;
-    if constexpr (BGK) collide_bgk_x<C, RatesC<C>, TQ>(r, f, t);
+    if constexpr (BGK) collide_bgk_x<C, R, TQ>(r, f, t);
     else if constexpr (sizeof(C) == 8 && TQ == 5) collide_d(r, f, t);
+    else if constexpr (std::is_same<R, RatesHalf9>::value) collide_u<C>(r, f, t);
     else collide_x<C, TQ>(r, f, t);
 }
 
 // Collide cells K and K + 1 of an N-cell group as one float2 pair, in place.
-template <int K, int N, int TQ = 5, bool BGK = false>
-__device__ __forceinline__ void collide_pair(const RatesC<float> &r, float f[9][N], float t[TQ][N]) {
+template <int K, int N, int TQ = 5, bool BGK = false, typename R>
+__device__ __forceinline__ void collide_pair(const R &r, float f[9][N], float t[TQ][N]) {
     float2 fp[9], tp[TQ];
 #pragma unroll
     for (int i = 0; i < 9; ++i) fp[i] = make_float2(f[i][K], f[i][K + 1]);
 #pragma unroll
     for (int i = 0; i < TQ; ++i) tp[i] = make_float2(t[i][K], t[i][K + 1]);
-    if constexpr (BGK) collide_bgk_x<float2, RatesC<float>, TQ>(r, fp, tp);
+    if constexpr (BGK) collide_bgk_x<float2, R, TQ>(r, fp, tp);
+    else if constexpr (std::is_same<R, RatesHalf9>::value) collide_u<float2>(r, fp, tp);
     else collide_x<float2, TQ>(r, fp, tp);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -848,7 +985,8 @@ __device__ __forceinline__ void zero_solid(uint32_t mN, float f[9][N], float t[T
 // ------------------------------------------------------------------ kernels
 
 template <typename S, int TQ = 5, bool BGK = false>
-__global__ void __launch_bounds__(256) k_step(const Planes<S> pl, const Geom g, const RatesC<typename Store<S>::C> r) {
+__global__ void __launch_bounds__(256)
+    k_step(const Planes<S> pl, const Geom g, const typename StepRates<S, TQ, BGK, TQ == 9 && BGK>::type r) {
     using C = typename Store<S>::C;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.nx) return;
@@ -1352,8 +1490,8 @@ __device__ __forceinline__ void pull_from_right(const float a[4], float edge, in
 // One warp's share of a row: cells x0..x0+3 of row y for each lane (x0 = base +
 // 4 lane). Every lane of the warp calls it with the same y. PA gives the plane
 // pointers (Planes, or a batch member's).
-template <typename S, typename PA, bool NC = true, int TQ = 5, bool BGK = false>
-__device__ __forceinline__ void row4(const PA &pl, const Geom &g, const RatesC<float> &r, int x0, int y, int lane) {
+template <typename S, typename PA, bool NC = true, int TQ = 5, bool BGK = false, typename R>
+__device__ __forceinline__ void row4(const PA &pl, const Geom &g, const R &r, int x0, int y, int lane) {
     const int r0 = y * g.pitch;
     const bool inrow = x0 < g.pitch;
     uint32_t m4 = 0xFFFFFFFFu;
@@ -1525,7 +1663,9 @@ struct PrefetchRows {
 // and its writes are visible, before its first global access. Launched without
 // that attribute, the wait returns at once.
 template <typename S, int MINB, int TQ = 5, bool BGK = false>
-__global__ void __launch_bounds__(128, MINB) k_step4(const Planes<S> pl, const Geom g, const RatesC<float> r) {
+__global__ void __launch_bounds__(128, MINB)
+    k_step4(const Planes<S> pl, const Geom g,
+            const typename StepRates<S, TQ, BGK, MINB <= (sizeof(S) == 2 ? 4 : 5)>::type r) {
     constexpr int PF = PrefetchRows<S>::value;
     constexpr int MPF = PrefetchRows<S>::mask;
     static_assert(PF == 0 || PF == MPF, "FP16 prefetches planes and link map with one lead");
@@ -1566,7 +1706,8 @@ __global__ void __launch_bounds__(128, MINB) k_step4(const Planes<S> pl, const G
 // with a prefetch per warp). Same row code, same bits; launched like k_step4.
 template <typename S, int MINB, int TQ = 5, bool BGK = false>
 __global__ void __launch_bounds__(128, MINB)
-    k_step4w(const Planes<S> pl, const Geom g, const RatesC<float> r, int upr, int nunits) {
+    k_step4w(const Planes<S> pl, const Geom g, const typename StepRates<S, TQ, BGK, sizeof(S) == 4 && MINB <= 7>::type r,
+             int upr, int nunits) {
     constexpr int PF = PrefetchRows<S>::value;
     constexpr int MPF = PrefetchRows<S>::mask;
     static_assert(PF == 0 || PF == MPF, "FP16 prefetches planes and link map with one lead");
