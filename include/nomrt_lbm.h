@@ -163,7 +163,8 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
 /* Advance nsteps >= 0 time steps (Eqs. 8-9 and 24-25, fused). Asynchronous on the
  * lattice's stream. With the AUTO step kernel, runs of two steps or more of an
  * FP32 or FP16 lattice without node-based walls (and with at most 15 walls; in
- * FP16 up to 6.5 million cells, 4 million with nine temperature populations) take
+ * FP16 up to 6.5 million cells, 4 million with nine temperature populations, for
+ * runs of two steps 5 and 0.9 million) take
  * up to eight steps per launch, tile by tile in shared memory, the tile and the
  * steps per launch chosen from the lattice's size, unless that says that single
  * steps are faster (wide lattices of few rows); the bits are those of single

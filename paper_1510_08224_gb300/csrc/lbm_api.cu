@@ -963,7 +963,8 @@ lbm_status lbm_step(lbm_lattice *h, int64_t nsteps) {
     const cudaError_t ce = cudaStreamIsCapturing(h->stream, &cs);
     if (ce != cudaSuccess) cudaGetLastError();  // leave no error behind for the launch checks
     if (ce == cudaSuccess && cs != cudaStreamCaptureStatusNone) h->recorded = true;
-    if (nsteps > 1 && h->kp.variant == nomrt::kStepAuto && plan_tiles(h)) return step_tiles(h, nsteps);
+    if (nsteps > 1 && h->kp.variant == nomrt::kStepAuto && plan_tiles(h) && nsteps >= h->tile_plan.least)
+        return step_tiles(h, nsteps);
     const bool can_graph = !h->graph_off && ce == cudaSuccess && cs == cudaStreamCaptureStatusNone;
     if (!can_graph || nsteps < kGraphShort) return step_direct(h, nsteps);
     if (!h->direct_done || h->graph_variant != h->kp.variant || h->graph_config != h->kp.config) {

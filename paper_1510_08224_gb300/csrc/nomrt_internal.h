@@ -108,10 +108,10 @@ struct KParams {
 };
 
 // How a lattice steps several times per launch: a tile shape (an index, -1: it
-// does not) and the steps per launch, and whether launches of one step each are
-// faster than single steps.
+// does not) and the steps per launch; the fewest steps of a run that takes the
+// tiles, and whether launches of one step each are faster than single steps.
 struct TilePlan {
-    int shape = -1, steps = 0;
+    int shape = -1, steps = 0, least = 2;
     bool one = false;
 };
 

@@ -109,15 +109,20 @@ inline double tile_share(const KParams *const *lats, int n, int elem) {
 constexpr int kTileMaxSteps = 8;
 constexpr double kL2Bytes = 100e6;  // what of the 129 MB L2 two buffers can count on
 
-// Cells up to which one FP16 lattice takes several steps per launch. A block
-// keeps FP32 images, so it computes as long as an FP32 lattice's and rounds
+// Cells up to which a run of `steps` steps of one FP16 lattice takes the tiles. A
+// block keeps FP32 images, so it computes as long as an FP32 lattice's and rounds
 // every population besides, while single steps are bound by HBM at half the
 // bytes. Measured, us per step, single -> several steps per launch: 1024^2 14.1
 // -> 12.0, 2048 x 1024 24.5 -> 20.2, 2500^2 59.8 -> 57.5, 4096 x 2048 72.6 ->
 // 74.3; with nine temperature populations 1777^2 49.3 -> 43.5, 4096 x 1024 53.9
-// -> 55.1. A batch's single steps are further from that bound (64 lattices of
-// 300^2: 120 -> 76) and have no such limit.
-inline double tile_most_f16(int nq) { return nq <= 14 ? 6.5e6 : 4.0e6; }
+// -> 55.1. Runs of two steps: 1402^2 26.3 -> 23.4, 2050^2 46.0 -> 44.5, 2450^2 59.9
+// -> 60.8; with nine 802^2 13.9 -> 13.7, 1026^2 19.2 -> 19.9. A batch's single
+// steps are further from that bound (64 lattices of 300^2: 120 -> 76) and have no
+// such limit.
+inline double tile_most_f16(int nq, int steps) {
+    if (nq <= 14) return steps == 2 ? 5.0e6 : 6.5e6;
+    return steps == 2 ? 0.9e6 : 4.0e6;
+}
 
 // The shape and steps per launch with the least estimated time per step, or shape
 // -1 where single steps are estimated faster. Lattices with node-based walls or more walls than a block keeps step once per
@@ -136,7 +141,7 @@ inline TilePlan choose_tile(const KParams *const *lats, int n, bool batch, int n
         if (p.n_nee > 0 || p.n_walls > kTileWalls || (!batch && (c.rows <= 0 || c.cols <= 0))) return best;
         cells += (double)p.nx * p.ny;
     }
-    if (elem == 2 && !batch && cells > tile_most_f16(nq)) return best;
+    if (elem == 2 && !batch && cells > tile_most_f16(nq, kTileMaxSteps)) return best;
     const double cell_bytes = 2.0 * nq * elem;
     const bool fits_l2 = cell_bytes * cells < kL2Bytes;
     // tiles of a launch of k steps (-1: more than a launch can have)
@@ -169,6 +174,7 @@ inline TilePlan choose_tile(const KParams *const *lats, int n, bool batch, int n
     if (best.shape < 0) return best;
     const double single = single_cycles(lats, n, nq, elem, sms);
     if (least > tile_share(lats, n, elem) * single) return TilePlan{};
+    if (elem == 2 && !batch && cells > tile_most_f16(nq, 2)) best.least = 3;
     // launches of one step (two steps that have to end on the buffer they began on): by the same estimates, or
     // up to one wave of tiles, FP16 two, where single steps launched one by one take longer than replayed (24
     // lattices of 32 to 128: 7.7 us a step against 10.2; 8 of 200 to 400, 1.8 waves, FP32 14.8 / 14.4, FP16 14.9

@@ -81,3 +81,9 @@ def test_two_steps_that_end_on_their_first_buffer(side, storage):
         for u, v in zip(lat.populations(), want):
             assert np.array_equal(u, v)
     batch.close()
+
+
+def test_two_steps_of_a_large_half_precision_lattice():
+    """Single steps for a run of two, the tiles for longer ones."""
+    case = lc.with_d2q9_temperature(lc.cavity(n=1001, n_y=990, Ra=1e5, noise=1e-3))
+    assert _same_as_single_steps(case, "f16", (2, 3, 8)) > 1
