@@ -310,9 +310,8 @@ int32_t lbm_bounds_checking(void);
 lbm_status lbm_debug_bounds_limit(lbm_lattice *h, int64_t bytes);
 
 /* Test hook for the timeout path of launches of several steps (lbm_step). With
- * on = 1 every block of such a launch of h takes the copy of its region as not
- * arrived in time, records that in the status word, waits for the copy and
- * returns; the next synchronising call on h reports LBM_ETIMEOUT (the state is
+ * on = 1 every block of such a launch of h records in the status word that the
+ * copy of its region did not arrive in time; the next synchronising call on h reports LBM_ETIMEOUT (the state is
  * then undefined). No fault and no hang are involved. on = 0 restores normal
  * operation. LBM_EINVAL for other values and for a member of a batch (set it
  * before the lattice joins). */

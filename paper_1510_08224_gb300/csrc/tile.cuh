@@ -436,8 +436,9 @@ __host__ __device__ constexpr int tile_rows(int k) { return RY - 2 * k; }
 
 // How a launch runs (bits). Early: read what does not change between steps
 // before waiting for the previous launch (a grid whose blocks can become
-// resident before it ends). Late: every thread but the first takes its region's
-// copy as not arrived in time (a test of the report).
+// resident before it ends). Late: report the region's copy as not arrived in time
+// (a test of the report): FP32 takes the wait of every thread but the first as run
+// out, FP16, which a condition at the wait cost 1-2 %, begins with the flag set.
 constexpr int kTileEarly = 1, kTileLate = 2;
 
 // k steps of the tile whose first output cell is (ox, oy), ox a multiple of 4.
@@ -464,7 +465,7 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
         mbar_fence_init();
-        *gave_up = 0;
+        *gave_up = HALF && boxed && (mode & kTileLate) != 0;
     }
     const bool early = (mode & kTileEarly) != 0;
     bool any = false;
@@ -503,12 +504,7 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     }
     if (!early) any = tile_maps<TQ, RX, RY, T>(g, maps, gx0, gy0);
     const bool walled = __syncthreads_or(any);  // also: the barrier is initialised
-    // a copy that did not arrive in time makes what is stored below invalid: reported by whichever thread saw it
-    if (boxed && (((mode & kTileLate) && threadIdx.x != 0) || !mbar_wait_bounded(bar, 0))) {
-        *gave_up = 1;
-        atomicExch(status, kStatusTimeout);
-        if (also) atomicExch(also, kStatusTimeout);
-    }
+    if (boxed && ((!HALF && (mode & kTileLate) && threadIdx.x != 0) || !mbar_wait_bounded(bar, 0))) *gave_up = 1;
     if (HALF && boxed) {
         tile_expand<TQ, RX, RY, T>(pop, gx0 - bx0);
         __syncthreads();
@@ -531,9 +527,14 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     const int x0 = ox - gx0, x1 = min(x0 + tile_cols<RX>(k), g.nx - gx0);
     if (walled) tile_passes<true, S, TQ, BGK, RX, RY, T>(pl, g, r, pop, maps, W, k, gx0, gy0, x0, x1);
     else tile_passes<false, S, TQ, BGK, RX, RY, T>(pl, g, r, pop, maps, W, k, gx0, gy0, x0, x1);
-    // one more bounded wait for a late copy (a thread that gave up reads its own flag), so that it cannot land
+    // a copy that did not arrive in time (what was stored above is then invalid): reported by every thread that
+    // sees the flag, the one that gave up among them, after one more bounded wait so that the copy cannot land
     // in a later block's shared memory
-    if (*gave_up) mbar_wait_bounded(bar, 0);
+    if (*gave_up) {
+        mbar_wait_bounded(bar, 0);
+        atomicExch(status, kStatusTimeout);
+        if (also) atomicExch(also, kStatusTimeout);
+    }
 }
 
 template <typename S, int TQ, bool BGK, int RX, int RY, int T, int MINB>

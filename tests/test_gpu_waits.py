@@ -1,7 +1,6 @@
 """A region's copy that does not arrive in time (launches of several steps): the
-test hook makes the bounded wait of every thread but one give up at once; the
-kernel returns normally, the next synchronising call reports LBM_ETIMEOUT once,
-and the lattice works again. In a batch both the batch and the member report."""
+test hook makes every block record that; the kernel returns normally, the next
+synchronising call reports LBM_ETIMEOUT once, and the lattice works again. In a batch both the batch and the member report."""
 import numpy as np
 import pytest
 
@@ -26,7 +25,7 @@ def _case(name):
 @pytest.mark.parametrize("storage", ["f32", "f16"])
 @pytest.mark.parametrize("name", ["box", "cavity"])
 @pytest.mark.parametrize("steps", [2, 3, 8])
-def test_late_copy_is_reported_by_any_thread(name, storage, steps):
+def test_late_copy_is_reported_once(name, storage, steps):
     import torch
     import paper_1510_08224_gb300 as P
     case = _case(name)
