@@ -560,7 +560,6 @@ void plan_tiles(lbm_batch *b) {
             std::memset(&t, 0, sizeof t);
             t.rc = G.rc;
             t.nlats = G.nlats;
-            t.status = b->d_status;
         }
         for (int m = 0; m < G.nlats; ++m) {
             const lbm_lattice *h = b->members[b->member_of[gi * nomrt::kGroupLats + m]];
@@ -581,8 +580,7 @@ void plan_tiles(lbm_batch *b) {
                 t.plane = h->kp.plane;
                 t.v = G.lat[m].v;
                 t.walls = nomrt::TileWalls{h->kp.n_walls, h->kp.moving};
-                t.status = h->kp.status;
-                t.late = h->kp.late ? nomrt::kTileLate : 0;
+                t.report = nomrt::TileReport{h->kp.status, b->d_status, h->kp.late};
                 t.row0 = h->kp.py ? 0 : 1;
             }
         }

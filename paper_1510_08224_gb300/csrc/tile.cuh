@@ -437,17 +437,25 @@ __host__ __device__ constexpr int tile_rows(int k) { return RY - 2 * k; }
 // How a launch runs (bits). Early: read what does not change between steps
 // before waiting for the previous launch (a grid whose blocks can become
 // resident before it ends). Late: report the region's copy as not arrived in time
-// (a test of the report): FP32 takes the wait of every thread but the first as run
-// out, FP16, which a condition at the wait cost 1-2 %, begins with the flag set.
+// (a test of the report): a single FP32 lattice takes the wait of every thread but
+// the first as run out; FP16 and batches, which a condition at the wait cost 1-2 %,
+// begin with the flag set.
 constexpr int kTileEarly = 1, kTileLate = 2;
 
+// Where a late copy is reported: a status word and another (a batch's beside its
+// member's), or NULL; and whether this lattice's copies are the late ones. Read
+// only where they are needed.
+struct TileReport {
+    int *status, *also;
+    int late;
+};
+
 // k steps of the tile whose first output cell is (ox, oy), ox a multiple of 4.
-// map: the source buffer's tensor map. status: the word a late copy is reported
-// to; also: another, or NULL (a batch's beside its member's).
+// map: the source buffer's tensor map.
 template <typename S, int TQ, bool BGK, int RX, int RY, int T, typename PA>
 __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const RatesC<float> &r, TileWalls walls,
-                                           const CUtensorMap *map, int k, int ox, int oy, int mode, int *status,
-                                           int *also = nullptr) {
+                                           const CUtensorMap *map, int k, int ox, int oy, int mode,
+                                           const TileReport &rep) {
     using Lay = TileLayout<TQ, RX, RY>;
     extern __shared__ __align__(128) float tile_smem[];
     uint64_t *const bar = reinterpret_cast<uint64_t *>(tile_smem);
@@ -459,13 +467,13 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     const TileWall W{wall_tab, walls.moving != 0};
     // every region but one that wraps along y is copied through the tensor map (a copy starts on 16 bytes)
     const bool boxed = !(g.py && (gy0 < 0 || gy0 + RY > g.ny));
-    constexpr bool HALF = sizeof(S) == 2;
+    constexpr bool HALF = sizeof(S) == 2, PRESET = HALF || !std::is_same<PA, Planes<S>>::value;
     static_assert(!HALF || RX % 8 == 0, "a box row is whole 16-byte pieces");
     const int bx0 = HALF ? gx0 & ~7 : gx0;
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
         mbar_fence_init();
-        *gave_up = HALF && boxed && (mode & kTileLate) != 0;
+        *gave_up = PRESET && boxed && (mode & kTileLate) != 0 && rep.late != 0;
     }
     const bool early = (mode & kTileEarly) != 0;
     bool any = false;
@@ -504,7 +512,7 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     }
     if (!early) any = tile_maps<TQ, RX, RY, T>(g, maps, gx0, gy0);
     const bool walled = __syncthreads_or(any);  // also: the barrier is initialised
-    if (boxed && ((!HALF && (mode & kTileLate) && threadIdx.x != 0) || !mbar_wait_bounded(bar, 0))) *gave_up = 1;
+    if (boxed && ((!PRESET && (mode & kTileLate) && rep.late && threadIdx.x != 0) || !mbar_wait_bounded(bar, 0))) *gave_up = 1;
     if (HALF && boxed) {
         tile_expand<TQ, RX, RY, T>(pop, gx0 - bx0);
         __syncthreads();
@@ -532,8 +540,8 @@ __device__ __forceinline__ void tile_steps(const PA &pl, const Geom &g, const Ra
     // in a later block's shared memory
     if (*gave_up) {
         mbar_wait_bounded(bar, 0);
-        atomicExch(status, kStatusTimeout);
-        if (also) atomicExch(also, kStatusTimeout);
+        atomicExch(rep.status, kStatusTimeout);
+        if (rep.also) atomicExch(rep.also, kStatusTimeout);
     }
 }
 
@@ -543,7 +551,8 @@ __global__ void __launch_bounds__(T, MINB)
            TileWalls walls, int k, int row0, int mode, int *status) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     tile_steps<S, TQ, BGK, RX, RY, T>(pl, g, r, walls, &map, k, (int)blockIdx.x * tile_cols<RX>(k),
-                                      row0 + (int)blockIdx.y * tile_rows<RY>(k), mode, status);
+                                      row0 + (int)blockIdx.y * tile_rows<RY>(k), mode,
+                                      TileReport{status, nullptr, 1});
 }
 
 }  // namespace nomrt

@@ -49,8 +49,7 @@ struct TileMember {
     unsigned long long plane;  // elements per plane
     MemberRates v;
     TileWalls walls;
-    int *status;        // the member's status word
-    int late;           // kTileLate or 0
+    TileReport report;  // the member's status word and the batch's
     int row0;           // first row of the member's tiles
     int tiles_x;        // tiles per row of tiles
 };
@@ -59,9 +58,8 @@ struct TileGroup {
     RatesC<float> rc;   // rates shared by the group
     int nlats;
     int k;              // steps of this launch
-    int mode;           // kTileEarly or 0
+    int mode;           // kTileEarly, kTileLate
     int first[kGroupLats + 1];  // first tile of each member; first[nlats]: tiles of the launch
-    int *status;        // the batch's status word
     TileMember lat[kGroupLats];
 };
 static_assert(sizeof(TileGroup) <= 32764, "a launch group's descriptors must fit the kernel parameter space");
@@ -93,7 +91,7 @@ __global__ void __launch_bounds__(T, MINB) k_tile_batch(const __grid_constant__ 
     RatesC<float> r = P.rc;  // shared rates: parameter-bank operands
     apply_member(r, L.v);
     tile_steps<S, 5, false, RX, RY, T>(pl, g, r, L.walls, &L.map, P.k, bx * tile_cols<RX>(P.k),
-                                       L.row0 + by * tile_rows<RY>(P.k), P.mode | L.late, L.status, P.status);
+                                       L.row0 + by * tile_rows<RY>(P.k), P.mode, L.report);
 }
 
 // The several-steps-per-launch kernels of a batch (MRT, D2Q5).
@@ -143,6 +141,8 @@ struct TileBatchSet<S, ShapeOf<RX, RY, T, MINB>...> {
         if (at == 0) return cudaSuccess;
         G.k = k;
         G.mode = at <= (long long)sms * s.per_sm ? kTileEarly : 0;
+        for (int m = 0; m < G.nlats; ++m)
+            if (G.lat[m].report.late) G.mode |= kTileLate;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)at);
         cfg.blockDim = dim3(s.threads);
