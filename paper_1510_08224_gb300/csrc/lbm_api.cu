@@ -905,8 +905,9 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
     // a double's boundary (or T0 everywhere), else in row chunks through the staging area, which holds nq rows of
     // populations and so stage_rows * nq rows of T. Stream order keeps a chunk's upload behind
     // the previous chunk's init kernel; one wait at the end covers the host buffers.
-    const bool T_aligned = (uintptr_t)p->T_init % alignof(double) == 0;
-    const double *Tv = p->T_init && T_aligned ? static_cast<const double *>(device_view(p->T_init)) : nullptr;
+    const double *Tv = p->T_init ? static_cast<const double *>(device_view(p->T_init)) : nullptr;
+    const cudaMemcpyKind T_kind = Tv ? cudaMemcpyDefault : cudaMemcpyHostToDevice;  // may be device memory
+    if ((uintptr_t)p->T_init % alignof(double) != 0) Tv = nullptr;
     if (!p->T_init || Tv) {
         for (int r0 = 0; r0 < ny; r0 += 65535) {
             const int r1 = std::min(ny, r0 + 65535);
@@ -919,7 +920,7 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
         for (int r0 = 0; r0 < ny; r0 += t_rows) {
             const int r1 = std::min(ny, r0 + t_rows);
             if ((e = cudaMemcpyAsync(h->stage(), p->T_init + (size_t)r0 * nx, (size_t)(r1 - r0) * nx * sizeof(double),
-                                     cudaMemcpyDefault, st)) != cudaSuccess)
+                                     T_kind, st)) != cudaSuccess)
                 return cuda_bail(e, "upload T_init");
             if ((e = h->L->init_rows(kp, 0, r0, r1, h->stage(), st)) != cudaSuccess)
                 return cuda_bail(e, "init kernel");
@@ -1035,12 +1036,16 @@ lbm_status lbm_read_macro_rows(lbm_lattice *h, int32_t y0, int32_t y1, double *r
     // host memory where it shares the host's page tables; any other, and one that is not on a double's
     // boundary (the kernel stores whole doubles), sends every output through the staging area
     double *direct[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaMemcpyKind kind[4] = {cudaMemcpyDeviceToHost, cudaMemcpyDeviceToHost, cudaMemcpyDeviceToHost,
+                              cudaMemcpyDeviceToHost};
     bool in_place = true;
     for (int k = 0; k < 4; ++k)
         if (outs[k]) {
             const bool aligned = (uintptr_t)outs[k] % alignof(double) == 0;
-            if (aligned) direct[k] = static_cast<double *>(const_cast<void *>(device_view(outs[k])));
-            if (aligned && !direct[k] && reaches_host() && map_pages(outs[k], (size_t)(y1 - y0) * nx * sizeof(double)))
+            direct[k] = static_cast<double *>(const_cast<void *>(device_view(outs[k])));
+            if (direct[k]) kind[k] = cudaMemcpyDefault;  // may be device memory
+            if (!aligned) direct[k] = nullptr;
+            else if (!direct[k] && reaches_host() && map_pages(outs[k], (size_t)(y1 - y0) * nx * sizeof(double)))
                 direct[k] = outs[k];
             in_place = in_place && direct[k];
         }
@@ -1073,7 +1078,7 @@ lbm_status lbm_read_macro_rows(lbm_lattice *h, int32_t y0, int32_t y1, double *r
                 if (outs[k])
                     LBM_CUDA(h,
                              cudaMemcpyAsync(outs[k] + (size_t)(r0 - y0) * nx, h->stage() + k * n, n * sizeof(double),
-                                             cudaMemcpyDefault, h->stream),
+                                             kind[k], h->stream),
                              "read macro");
         }
     }
