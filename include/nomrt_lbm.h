@@ -168,9 +168,8 @@ lbm_status lbm_create(const lbm_params *p, void *cuda_stream, void *device_mem, 
  * up to eight steps per launch, tile by tile in shared memory, the tile and the
  * steps per launch chosen from the lattice's size, unless that says that single
  * steps are faster (wide lattices of few rows); the bits are those of single
- * steps. Every other step is one kernel,
- * plus one for the boundary nodes of node-based walls; runs of 4 such steps or
- * more replay CUDA graphs of 32 and of 4 steps, captured once per step-kernel
+ * steps. Every other step is one kernel, in FP32 and FP16 plus one for the
+ * boundary nodes of node-based walls; runs of 4 such steps or more replay CUDA graphs of 32 and of 4 steps, captured once per step-kernel
  * choice (the same kernels and bits, without the launch gap between steps; a
  * step launched directly first where the graphs' starting buffer needs it);
  * shorter runs and the remainder, and calls on a stream that is being captured,
@@ -186,10 +185,11 @@ lbm_status lbm_sync(lbm_lattice *h);
 
 /* Step kernel variants. All compute the same arithmetic and give the same
  * bits for a given storage. AUTO picks the fastest measured on GB300: several
- * steps per launch where lbm_step says so, and for single steps the scalar
- * kernel for FP64, VEC4 for FP32 / FP16 with config 1 / 1 (MRT, D2Q5),
- * 0 / 1 (BGK, D2Q5) or 0 / 0 (D2Q9 temperature model), except VEC4W config 1
- * for FP32 MRT D2Q5 lattices whose rows are not a multiple of 512 cells.
+ * steps per launch where lbm_step says so, and for single steps one cell per
+ * thread for FP64 (boundary nodes in the same launch), VEC4 for FP32 / FP16 with
+ * config 1 / 1 (MRT, D2Q5), 0 / 1 (BGK, D2Q5) or 0 / 0 (D2Q9 temperature model),
+ * except VEC4W config 1 for FP32 MRT D2Q5 lattices whose rows are not a multiple
+ * of 512 cells.
  * SCALAR: one cell per thread. VEC4: four cells per thread with 128-bit (FP32)
  * / 64-bit (FP16) loads and warp shuffles for the x +- 1 pulls, one 512-cell
  * row segment per 128-thread block; configs 0-4 ask for 4, 5, 6, 7 or 8
@@ -222,7 +222,8 @@ int32_t lbm_step_kernel_count(int32_t storage, int32_t variant);
 lbm_status lbm_set_step_kernel(lbm_lattice *h, int32_t variant, int32_t config);
 
 /* Macroscopic fields into caller-owned host arrays of ny*nx doubles (any may be
- * NULL): the values the next collision would use (pull with the wall rules,
+ * NULL; on any byte: those on a double's boundary that the GPU reaches are written
+ * in place, others through the staging area): the values the next collision would use (pull with the wall rules,
  * then rho = sum f_bar (Eq. 18), rho0 u = sum e f_bar + F/2 (Eq. 19),
  * T = sum g (Eq. 27)). Solid cells read 0. Synchronises. */
 lbm_status lbm_read_macro(lbm_lattice *h, double *rho, double *ux, double *uy, double *T);

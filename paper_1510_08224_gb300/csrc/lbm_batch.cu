@@ -419,7 +419,7 @@ cudaError_t launch_batch_persistent(int config, const GroupParams &G, int parity
 // The residuals of up to kGroupLats members in one launch: each member's blocks and
 // sums are those of lbm_residual (residual_cells, reduce_finish), so its value
 // has the same bits. Measured against one kernel pair per member: 24 lattices of
-// 32 to 128, 640 -> 43 us; 64 of 128 to 1024, 3.1 -> 1.18 ms (the members' many
+// 32 to 128, 640 -> 44 us; 64 of 128 to 1024, 3.1 -> 1.16 ms (the members' many
 // small blocks; fewer, longer ones would take 0.73 ms, but a member's sums would
 // then depend on its batch).
 struct ResidualMember {

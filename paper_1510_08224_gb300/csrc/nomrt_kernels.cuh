@@ -275,7 +275,7 @@ inline Geom make_geom(const KParams &p) {
 // lattice's bounds word, which the synchronising calls report; nothing traps.
 // The sites: 1-9 pull / scalar kernel, 10-19 four-cell rows, 20-29 wall
 // links and node pass, 30-39 eight-cell kernel, 40-49 TMA kernel, 50-59
-// prefetches. Without LBM_BOUNDS every check is the constant true.
+// prefetches, 60-64 tiles. Without LBM_BOUNDS every check is the constant true.
 #ifdef LBM_BOUNDS
 static __device__ __noinline__ void oob_note(int *w, int site) { atomicCAS(w, 0, site); }
 

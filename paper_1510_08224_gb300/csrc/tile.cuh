@@ -50,7 +50,7 @@
 // (0.56 to 0.81 cycles); alone they run at 0.75 cells per cycle and SM, in
 // place at 0.66. Small lattices are bound by the latency of a step (about 1300
 // cycles) and of a launch. Measured, us per step, one step per launch -> this:
-// FP32 4096 x 2048 138 -> 60, 1024^2 22 -> 11, 600^2 7.0 -> 5.8, 128^2 5.5 ->
+// FP32 4096 x 2048 138 -> 60, 1024^2 22 -> 11, 600^2 7.0 -> 5.1, 128^2 5.5 ->
 // 1.4, 64^2 5.9 -> 1.2; with the D2Q9 temperature model 177 -> 88 at 4096 x
 // 2048; FP16 2048 x 1024 24.5 -> 20.2, 1024^2 14.1 -> 12.0, 600^2 9.1 -> 5.7,
 // 128^2 5.8 -> 1.5.

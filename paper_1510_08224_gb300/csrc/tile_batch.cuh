@@ -4,9 +4,9 @@
 // (found by a binary search over the members' first tiles) and the rates shared
 // by the group are block-uniform operands.
 // Bound as k_tile is. Measured, us per step, one step per launch -> this: 64
-// cavities of sides 128 to 1024 436 -> 204 (FP16 374 -> 239; with the members'
-// own kernels side by side 448 and 298), 24 of 32 to 128 7.3 -> 4.3, 64 FP16
-// lattices of 300^2 120 -> 76.
+// cavities of sides 128 to 1024 434 -> 204 (FP16 350 -> 258; with the members'
+// own kernels side by side 448 and 298), 24 of 32 to 128 7.2 -> 4.3 (FP16 13.6 ->
+// 5.1), 64 cavities of 300^2 119 -> 57 (FP16 105 -> 71).
 #pragma once
 
 #include "tile_launch.cuh"

@@ -37,7 +37,9 @@ inline TileCover tile_cover(const KParams &p) {
 // constants are a least-squares fit to 551 timed launches of 16 shapes with 2
 // to 8 steps on lattices of 64^2 to 4096 x 2048 cells and on batches of 24 to
 // 64 cavities (rms error 13 %); the shape and steps it picks run within 2 % of
-// the fastest of them but for 180^2 cells (19 %).
+// the fastest of them but for 180^2 cells (19 %). Fitted in FP32, before the next
+// block's prefetch went and before FP16's regions came through the tensor map:
+// FP16's conversions are not in it.
 inline double tile_cycles(const TileShape &s, int k, long long tiles, int nq, double cell_bytes, bool fits_l2,
                           int sms) {
     constexpr double kLaunch = 11600, kRound = 1.18;
@@ -117,7 +119,7 @@ constexpr double kL2Bytes = 100e6;  // what of the 129 MB L2 two buffers can cou
 // 74.3; with nine temperature populations 1777^2 49.3 -> 43.5, 4096 x 1024 53.9
 // -> 55.1. Runs of two steps: 1402^2 26.3 -> 23.4, 2050^2 46.0 -> 44.5, 2450^2 59.9
 // -> 60.8; with nine 802^2 13.9 -> 13.7, 1026^2 19.2 -> 19.9. A batch's single
-// steps are further from that bound (64 lattices of 300^2: 120 -> 76) and have no
+// steps are further from that bound (64 lattices of 300^2: 105 -> 71) and have no
 // such limit.
 inline double tile_most_f16(int nq, int steps) {
     if (nq <= 14) return steps == 2 ? 5.0e6 : 6.5e6;
